@@ -1,6 +1,7 @@
 #include "engine.cuh"
 
 #include <cmath>
+#include <cstring>
 
 namespace tatrg {
 
@@ -180,7 +181,9 @@ Engine::MetricOrth Engine::orth_metric(const double* X, int64_t nin, int64_t w, 
 SvdResult Engine::svd(const double* A, int64_t m, int64_t n) {
   SvdResult r;
   const int64_t k = std::min(m, n);
-  r.S = DevBuf(k * sizeof(double), s_);
+  // the status word after the singular values: one read brings both
+  r.S = DevBuf((k + 1) * sizeof(double), s_);
+  int* const status = reinterpret_cast<int*>(r.S.d() + k);
   if (m >= n) {
     r.U.buf = dalloc(m * n, s_);
     r.U.rows = m;
@@ -188,8 +191,8 @@ SvdResult Engine::svd(const double* A, int64_t m, int64_t n) {
     r.V.buf = dalloc(n * n, s_);
     r.V.rows = n;
     r.V.cols = n;
-    if (qrcp_svd_fits(m, int(n))) jacobi_svd_qrcp(A, m, int(n), r.U.p(), r.S.d(), r.V.p(), flag(1), s_, &st_);
-    else jacobi_svd(A, m, int(n), r.U.p(), r.S.d(), r.V.p(), flag(1), s_, &st_);
+    if (qrcp_svd_fits(m, int(n))) jacobi_svd_qrcp(A, m, int(n), r.U.p(), r.S.d(), r.V.p(), status, s_, &st_);
+    else jacobi_svd(A, m, int(n), r.U.p(), r.S.d(), r.V.p(), status, s_, &st_);
   } else {
     DevBuf At(m * n * sizeof(double), s_);
     transpose(A, m, n, At.d(), s_);
@@ -199,12 +202,14 @@ SvdResult Engine::svd(const double* A, int64_t m, int64_t n) {
     r.U.buf = dalloc(m * m, s_);
     r.U.rows = m;
     r.U.cols = m;
-    if (qrcp_svd_fits(n, int(m))) jacobi_svd_qrcp(At.d(), n, int(m), r.V.p(), r.S.d(), r.U.p(), flag(1), s_, &st_);
-    else jacobi_svd(At.d(), n, int(m), r.V.p(), r.S.d(), r.U.p(), flag(1), s_, &st_);
+    if (qrcp_svd_fits(n, int(m))) jacobi_svd_qrcp(At.d(), n, int(m), r.V.p(), r.S.d(), r.U.p(), status, s_, &st_);
+    else jacobi_svd(At.d(), n, int(m), r.V.p(), r.S.d(), r.U.p(), status, s_, &st_);
   }
   r.r = int(k);
-  r.s = to_host(r.S.d(), k);
-  const int jst = read_flag(1);
+  r.s = to_host(r.S.d(), k + 1);
+  int jst = 0;
+  std::memcpy(&jst, &r.s[k], sizeof(int));
+  r.s.resize(k);
   TATRG_CHECK(jst != 2, TATRG_ETIMEOUT, "Jacobi SVD: a grid barrier timed out");
   TATRG_CHECK(jst == 0, TATRG_ENUMERIC, "Jacobi SVD did not converge");
   for (double x : r.s) TATRG_CHECK(std::isfinite(x), TATRG_ENUMERIC, "non-finite singular value");

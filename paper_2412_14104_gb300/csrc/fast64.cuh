@@ -1,0 +1,89 @@
+// Scalar float64 functions for the serial chains of the small factorisations.  On GB300 an
+// FP64 instruction holds a warp for 64 clocks whatever its active lanes; the library's
+// sqrt, division and 1/sqrt are dependent sequences of them (measured: 680, 420 and 370
+// clocks).  These take a float seed from the MUFU unit, with the exponents handled on the
+// integer pipe, and one third-order step in float64: 3 to 6 FP64 instructions, results
+// within about two units in the last place.  Arguments must be positive and normal.
+#pragma once
+
+#include <stdint.h>
+
+namespace tatrg {
+
+__device__ __forceinline__ int exponent_field(double x) {
+  return int((uint64_t(__double_as_longlong(x)) >> 52) & 0x7FF);
+}
+// a normal float times 2^shift, exact (integer pipe); the result must be a normal double
+__device__ __forceinline__ double f2d_shift(float f, int shift) {
+  const uint32_t u = __float_as_uint(f);
+  const uint64_t e = uint64_t(int((u >> 23) & 0xFFu) + 896 + shift);
+  return __longlong_as_double(int64_t((uint64_t(u & 0x80000000u) << 32) | (e << 52) | (uint64_t(u & 0x7FFFFFu) << 29)));
+}
+// x 2^(1023 - E) truncated to float: 0 below float's normal range, NaN above it
+__device__ __forceinline__ float d2f_scaled(double x, int E) {
+  const uint64_t b = uint64_t(__double_as_longlong(x));
+  const int e = int((b >> 52) & 0x7FF) - E + 127;
+  const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
+  if (e <= 0) return __uint_as_float(sign);
+  if (e >= 255) return __uint_as_float(0x7FC00000u);
+  return __uint_as_float(sign | (uint32_t(e) << 23) | (uint32_t(b >> 29) & 0x7FFFFFu));
+}
+
+// Power of two that brings a matrix whose largest entry has exponent field E near 1, so
+// that products of its entries stay normal; 1 when they do anyway (or when the matrix is
+// zero or not finite).  Multiplying by it and by its reciprocal is exact.
+__device__ __forceinline__ double range_scale(int E) {
+  if (E == 0 || E == 0x7FF || (E > 823 && E < 1223)) return 1.0;
+  return __longlong_as_double(int64_t(2046 - E) << 52);
+}
+
+// 1 / d (d normal, exponent field below 2044)
+__device__ __forceinline__ double fast_rcp(double d) {
+  const int E = exponent_field(d);
+  const double y = f2d_shift(__frcp_rn(d2f_scaled(d, E)), 1023 - E);
+  const double e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// 1 / sqrt(d)
+__device__ __forceinline__ double fast_rsqrt(double d) {
+  const int E = exponent_field(d), odd = (E & 1) ^ 1;  // d = m 2^(E - 1023 - odd), m in [1, 4)
+  const double y = f2d_shift(rsqrtf(d2f_scaled(d, E - odd)), (1023 - (E - odd)) / 2);
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Rotation of a pair of columns with squared norms al, be and inner product ga: the angle
+// t = tan of the smaller rotation that makes them orthogonal, c = 1 / sqrt(1 + t^2) and
+// s = c t.  No rotation (false) when a column lies at or below the floor or the inner
+// product is within tol of orthogonal.  The test and the first estimate of t are float
+// arithmetic on values scaled by the larger norm's exponent; one Newton step in float64
+// takes t to ~1e-14 and c, s to rounding: 11 FP64 instructions.
+__device__ __forceinline__ bool jacobi_rotation(double al, double be, double ga, double floor2, float tol,
+                                                double& c, double& s) {
+  // non-negative doubles compare as integers
+  const int64_t fl = __double_as_longlong(floor2), ia = __double_as_longlong(al), ib = __double_as_longlong(be);
+  const int E = int(uint64_t(ia > ib ? ia : ib) >> 52);
+  if (!(ia > fl && ib > fl) || E >= 0x7FF) return false;
+  const float gf = d2f_scaled(ga, E), ag = fabsf(gf);
+  if (!(ag > tol * sqrtf(d2f_scaled(al, E) * d2f_scaled(be, E)))) return false;
+  const double d = be - al;
+  const float df = d2f_scaled(d, E), h = 0.5f * df, ah = fabsf(h);
+  const float hi = fmaxf(ah, ag), q = fminf(ah, ag) / hi;
+  const float tf = gf / (h + copysignf(hi * sqrtf(fmaf(q, q, 1.0f)), h));
+  double t = 0.0;
+  if (fabsf(tf) >= 1.1754944e-38f) {
+    t = f2d_shift(tf, 0);
+    // root of ga t^2 + d t - ga
+    const float ff = d2f_scaled(fma(fma(ga, t, d), t, -ga), E);
+    const float dt = -ff / fmaf(2.0f * gf, tf, df);
+    if (fabsf(dt) >= 1.1754944e-38f) t += f2d_shift(dt, 0);
+  }
+  const double w = fma(t, t, 1.0);
+  const double y = f2d_shift(rsqrtf(d2f_scaled(w, 1023)), 0);
+  const double e = fma(-w * y, y, 1.0);
+  c = fma(y * e, fma(0.375, e, 0.5), y);
+  s = c * t;
+  return true;
+}
+
+}  // namespace tatrg

@@ -4,8 +4,10 @@
 // Gram eigenvectors, squeezer factors and core, re-split): one block in shared memory for
 // small problems, otherwise one cooperative grid with a block per column pair.
 
-#include "kernels.cuh"
+#include <cooperative_groups.h>
 
+#include "fast64.cuh"
+#include "kernels.cuh"
 
 namespace tatrg {
 namespace {
@@ -113,85 +115,156 @@ __global__ void __launch_bounds__(128) tri_inverse_kernel(const double* R, int n
   for (int i = lane; i < n; i += 32) X[int64_t(i) * n + c] = x[i];
 }
 
-// One-sided Jacobi SVD.  Ac: column-major m x N workspace (N = n rounded up to even, the
-// padding column is zero), Vc: column-major N x N initialised to the identity.  The m x N
-// columns are worked on in shared memory and written back at the end; V stays in global
-// memory (L2).
-__global__ void __launch_bounds__(1024) jacobi_kernel(double* Acg, int64_t m, int N, double* Vc,
-                                                      int max_sweeps, double tol, int* status) {
-  extern __shared__ double Ac[];
-  __shared__ int rotated;
-  __shared__ double fro2, wsum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int64_t e = threadIdx.x; e < m * N; e += blockDim.x) Ac[e] = Acg[e];
-  // Columns whose squared norm is below (4 eps)^2 ||A||_F^2 sit at the rounding floor:
-  // they are treated as converged, otherwise rounding in a large-small pair keeps the
-  // relative inner product above tol forever.
-  __syncthreads();
-  {
-    double acc = 0.0;
-    for (int64_t e = threadIdx.x; e < m * N; e += blockDim.x) acc = fma(Ac[e], Ac[e], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) wsum[warp] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += wsum[w];
-      fro2 = t;
-    }
+// Sums of three values over the G lanes of a group (G = 16 or 32), in every lane: the first
+// two steps of the butterfly carry the values in different lanes, which takes 5 or 6 FP64
+// additions in place of 12 or 15.
+template <int G>
+__device__ __forceinline__ void group_sum3(double& a, double& b, double& c) {
+  const unsigned full = 0xffffffffu;
+  const bool hi = threadIdx.x & (G / 2), q = threadIdx.x & (G / 4);
+  const double s1 = hi ? a : c, s2 = hi ? b : 0.0;
+  double x = hi ? c : a, y = hi ? 0.0 : b;
+  x += __shfl_xor_sync(full, s1, G / 2);
+  y += __shfl_xor_sync(full, s2, G / 2);
+  double v = q ? y : x;
+  v += __shfl_xor_sync(full, q ? x : y, G / 4);
+#pragma unroll
+  for (int o = G / 8; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+  a = __shfl_sync(full, v, 0, G);
+  b = __shfl_sync(full, v, G / 4, G);
+  c = __shfl_sync(full, v, G / 2, G);
+}
+
+// x / y from r = 1 / y: one corrected quotient, or the division itself where r overflows
+__device__ __forceinline__ double div_by(double x, double y, double r) {
+  if (exponent_field(y) < 8) return x / y;
+  const double q = x * r;
+  return fma(fma(-q, y, x), r, q);
+}
+
+// One-sided Jacobi SVD of a narrow row-major m x n matrix (N = n rounded up to even < 32),
+// one block, the columns of A and V in shared memory, the whole factorisation in one launch
+// (transposed load, sweeps, column norms, descending order, scaled output).
+//
+// Bound by FP64 latency: a round is a chain of about 30 FP64 instructions of 64 clocks
+// (inner products, their reduction, the rotation's scalars, the update).  So a column pair
+// has one group of G lanes (16 for m <= 16, which packs two pairs into a warp), the groups
+// of a round spread over the SM's four FP64 ports, the reduction is group_sum3 and the
+// scalars are jacobi_rotation's.  A 12 x 12 SVD took 600 us per call with one warp per
+// pair, V in L2 and library square roots and divisions; see jacobi_svd for this form.
+//
+// Columns whose squared norm is below (4 eps)^2 ||A||_F^2 sit at the rounding floor: they
+// are treated as converged, otherwise rounding in a large-small pair keeps the relative
+// inner product above tol forever.
+template <int G>
+__global__ void __launch_bounds__(512) jacobi_small_kernel(const double* A, int64_t m, int n, int N, double* U,
+                                                           double* S, double* V, int max_sweeps, float tol,
+                                                           int* status) {
+  extern __shared__ double Ac[];  // m x N, then V: N x N, both column-major
+  __shared__ double wsum[16], sig[32], inv[32];
+  __shared__ int rank_s[32], top[16];
+  double* const Vc = Ac + m * N;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  int E = 0;
+  for (int64_t e = tid; e < m * N; e += nt) {
+    const int64_t i = e / N;
+    const int j = int(e - i * N);
+    const double x = j < n ? A[i * n + j] : 0.0;
+    Ac[j * m + i] = x;
+    E = max(E, exponent_field(x));
   }
+  for (int e = tid; e < N * N; e += nt) Vc[e] = (e / N == e % N) ? 1.0 : 0.0;
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (lane == 0) top[warp] = E;
   __syncthreads();
+  for (int w = 0; w < (nt >> 5); ++w) E = max(E, top[w]);
+  const double scale = range_scale(E);
+  double acc = 0.0;
+  for (int64_t e = tid; e < m * N; e += nt) {
+    double x = Ac[e];
+    if (scale != 1.0) Ac[e] = x *= scale;
+    acc = fma(x, x, acc);
+  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) wsum[warp] = acc;
+  __syncthreads();
+  double fro2 = 0.0;
+  for (int w = 0; w < (nt >> 5); ++w) fro2 += wsum[w];
   const double floor2 = 7.9e-31 * fro2;
+  const int L = N - 1, k = tid / G, g = tid % G;
+  const bool active = k < N / 2;
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) rotated = 0;
-    __syncthreads();
-    for (int r = 0; r < N - 1; ++r) {
-      for (int k = warp; k < N / 2; k += nw) {
-        int p, q;
-        if (k == 0) { p = N - 1; q = r % (N - 1); }
-        else { p = (r + k) % (N - 1); q = (r + N - 1 - k) % (N - 1); }
-        double* ap = Ac + int64_t(p) * m;
-        double* aq = Ac + int64_t(q) * m;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int64_t i = lane; i < m; i += 32) {
-          double x = ap[i], y = aq[i];
+    int rotated = 0;
+    for (int r = 0; r < L; ++r) {
+      int p = r + k, q = r + L - k;
+      p -= p >= L ? L : 0;
+      q -= q >= L ? L : 0;
+      if (k == 0) { p = N - 1; q = r; }
+      double* const ap = Ac + int64_t(active ? p : 0) * m;
+      double* const aq = Ac + int64_t(active ? q : 0) * m;
+      double al = 0.0, be = 0.0, ga = 0.0, c, sn;
+      if (active) {
+        for (int64_t i = g; i < m; i += G) {
+          const double x = ap[i], y = aq[i];
           al = fma(x, x, al);
           be = fma(y, y, be);
           ga = fma(x, y, ga);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        if (al > floor2 && be > floor2 && fabs(ga) > tol * sqrt(al) * sqrt(be)) {
-          double zeta = (be - al) / (2.0 * ga);
-          double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-          for (int64_t i = lane; i < m; i += 32) {
-            double x = ap[i], y = aq[i];
-            ap[i] = c * x - s * y;
-            aq[i] = s * x + c * y;
-          }
-          double* vp = Vc + int64_t(p) * N;
-          double* vq = Vc + int64_t(q) * N;
-          for (int i = lane; i < N; i += 32) {
-            double x = vp[i], y = vq[i];
-            vp[i] = c * x - s * y;
-            vq[i] = s * x + c * y;
-          }
-          if (lane == 0) rotated = 1;
-        }
       }
-      __syncthreads();
+      group_sum3<G>(al, be, ga);
+      if (active && jacobi_rotation(al, be, ga, floor2, tol, c, sn)) {
+        for (int64_t i = g; i < m; i += G) {
+          const double x = ap[i], y = aq[i];
+          ap[i] = c * x - sn * y;
+          aq[i] = sn * x + c * y;
+        }
+        double* const vp = Vc + p * N;
+        double* const vq = Vc + q * N;
+        for (int i = g; i < N; i += G) {
+          const double x = vp[i], y = vq[i];
+          vp[i] = c * x - sn * y;
+          vq[i] = sn * x + c * y;
+        }
+        rotated = 1;
+      }
+      if (r + 1 < L) __syncthreads();
     }
-    __syncthreads();
-    if (!rotated) break;
-    __syncthreads();
+    if (!__syncthreads_or(rotated)) break;
   }
-  for (int64_t e = threadIdx.x; e < m * N; e += blockDim.x) Acg[e] = Ac[e];
-  if (threadIdx.x == 0) *status = (sweep >= max_sweeps) ? 1 : 0;
+  // column norms by the same groups (columns 2k, 2k + 1), ranks (ties by index), outputs
+  {
+    double a2 = 0.0, b2 = 0.0, z = 0.0;
+    if (active) {
+      const double* const ap = Ac + int64_t(2 * k) * m;
+      for (int64_t i = g; i < m; i += G) {
+        a2 = fma(ap[i], ap[i], a2);
+        b2 = fma(ap[m + i], ap[m + i], b2);
+      }
+    }
+    group_sum3<G>(a2, b2, z);
+    if (active && g < 2) sig[2 * k + g] = sqrt(g ? b2 : a2);
+  }
+  __syncthreads();
+  if (tid < n) {
+    int rk = 0;
+    for (int i = 0; i < n; ++i) rk += (sig[i] > sig[tid]) || (sig[i] == sig[tid] && i < tid);
+    rank_s[tid] = rk;
+    S[rk] = scale != 1.0 ? sig[tid] / scale : sig[tid];
+    inv[tid] = 1.0 / sig[tid];
+  }
+  __syncthreads();
+  for (int64_t e = tid; e < m * n; e += nt) {
+    const int64_t i = e / n;
+    const int j = int(e - i * n);
+    const double sj = sig[j];
+    U[i * n + rank_s[j]] = sj > 0.0 ? div_by(Ac[j * m + i], sj, inv[j]) : 0.0;
+  }
+  for (int e = tid; e < n * n; e += nt) {
+    const int i = e / n, j = e % n;
+    V[i * n + rank_s[j]] = Vc[j * N + i];
+  }
+  if (tid == 0) *status = (sweep >= max_sweeps) ? 1 : 0;
 }
 
 // Column norms (one block per column), descending ranks (ties by index) and the
@@ -501,6 +574,300 @@ timed_out:
   if (threadIdx.x == 0) atomicExch(status, 2);
 }
 
+// Columns on the move between the blocks of jacobi_ring_kernel: a double is two 8-byte
+// words, each 32 bits of data under a 32-bit tag, so a reader that sees both tags has the
+// value; no separate flag and no fence (one trip through L2 instead of two).
+__device__ __forceinline__ void put_tagged(ulonglong2* p, double x, uint32_t tag) {
+  const uint64_t b = uint64_t(__double_as_longlong(x)), t = uint64_t(tag) << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"((b & 0xffffffffull) | t),
+               "l"((b >> 32) | t)
+               : "memory");
+}
+__device__ __forceinline__ bool get_tagged(const ulonglong2* p, uint32_t tag, double& x) {
+  uint64_t lo, hi;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+  x = __longlong_as_double(int64_t((lo & 0xffffffffull) | (hi << 32)));
+  return uint32_t(lo >> 32) == tag && uint32_t(hi >> 32) == tag;
+}
+
+struct RingArgs {
+  const double* A;  // row-major m x n
+  int m, n, N;      // N: n rounded up to even; N / 2 blocks
+  double *U, *S, *V;
+  double *part, *sig;  // N partial sums of squares; N column norms
+  int* top;            // largest exponent field of A
+  int* rot;            // per sweep: some block rotated
+  unsigned* bar;       // grid_barrier's words
+  ulonglong2* ring;    // [2][N / 2][2][m + N] tagged doubles
+  int* status;         // zero on entry; 1 not converged within max_sweeps, 2 a wait ran out
+  int max_sweeps;
+  float tol;
+};
+
+// One-sided Jacobi SVD, 32 <= N <= 256 and m <= 128 EA, N <= 128 EV: one block of 128 threads
+// per column pair of the round-robin schedule, the pair's columns of A and V in registers.
+// Between rounds a column moves to the next block of a ring: block k's first column goes to
+// block k - 1 and its second to block k + 1 (block 0 keeps column N - 1, the last block's
+// second column becomes its first), so a block waits for two neighbours and not for the
+// grid.  Two buffers by the parity of the round suffice: a block can be at most one round
+// ahead of a neighbour, since it needs that neighbour's column.  A's columns are sent as
+// soon as they are rotated; V's wait, rotation and send follow while A's are under way.
+//
+// Bound by the chain of a round: about 30 FP64 instructions of 64 clocks on the busiest
+// warp and one trip through L2.  A grid barrier per round with the columns in L2 and the
+// rotation's scalars on one thread with library square roots and divisions took 7.5 us a
+// round (144 x 144: 1287 rounds, 10.4 ms); see jacobi_svd for this form.
+//
+// Every wait is bounded by g_barrier_limit_ns; a wait that runs out raises the abort flag
+// bar[2], which every other waiting block reads, and all blocks return with status 2.
+template <int EA, int EV>
+__global__ void __launch_bounds__(128) jacobi_ring_kernel(const RingArgs a) {
+  __shared__ double part_s[3][128], tot_s[3], sig_s[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m = a.m, n = a.n, N = a.N, L = N - 1, K = N / 2, k = blockIdx.x;
+  const int len = m + N;
+  const uint64_t limit = g_barrier_limit_ns;
+  volatile unsigned* const abort_flag = a.bar + 2;
+  // V's rows go round the warps in another order than A's, so that the warp with A's last
+  // partial chunk is not the one with V's
+  const int tv = (tid + 64) & 127;
+  double xs[EA], ys[EA], vx[EV], vy[EV];
+  int p = k == 0 ? N - 1 : k, q = k == 0 ? 0 : L - k;
+#pragma unroll
+  for (int e = 0; e < EA; ++e) {
+    const int i = tid + 128 * e;
+    xs[e] = (i < m && p < n) ? a.A[int64_t(i) * n + p] : 0.0;
+    ys[e] = i < m ? a.A[int64_t(i) * n + q] : 0.0;
+  }
+#pragma unroll
+  for (int e = 0; e < EV; ++e) {
+    const int i = tv + 128 * e;
+    vx[e] = i == p ? 1.0 : 0.0;
+    vy[e] = i == q ? 1.0 : 0.0;
+  }
+  // where the columns go, by the parity of the round they are for
+  const int last = K - 1;
+  auto slot = [&](int parity, int block, int which) {
+    return a.ring + (int64_t(parity * K + block) * 2 + which) * len;
+  };
+  const int p_to = k == 1 ? 0 : k - 1, p_slot = k == 1 ? 1 : 0;  // block 1's first column is block 0's second
+
+  // the chunk loops' warp-uniform bounds skip FP64 work on rows past the end
+  auto dots = [&](double& al, double& be, double& ga) {
+    al = be = ga = 0.0;
+#pragma unroll
+    for (int e = 0; e < EA; ++e)
+      if (32 * warp + 128 * e < m) {
+        al = fma(xs[e], xs[e], al);
+        be = fma(ys[e], ys[e], be);
+        ga = fma(xs[e], ys[e], ga);
+      }
+  };
+  // block totals of three values per thread: warps 0..2 take one value each
+  auto totals = [&](bool ok, double& al, double& be, double& ga) {
+    part_s[0][tid] = al;
+    part_s[1][tid] = be;
+    part_s[2][tid] = ga;
+    if (!__syncthreads_and(ok)) return false;
+    if (warp < 3) {
+      double v = (part_s[warp][lane] + part_s[warp][lane + 32]) + (part_s[warp][lane + 64] + part_s[warp][lane + 96]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) tot_s[warp] = v;
+    }
+    __syncthreads();
+    al = tot_s[0];
+    be = tot_s[1];
+    ga = tot_s[2];
+    return true;
+  };
+
+  auto advance = [&]() {  // the next round's columns (modulo the sweep)
+    p = k == 0 ? p : (p + 1 == L ? 0 : p + 1);
+    q = q + 1 == L ? 0 : q + 1;
+    if (k == last) {
+#pragma unroll
+      for (int e = 0; e < EA; ++e) xs[e] = ys[e];
+#pragma unroll
+      for (int e = 0; e < EV; ++e) vx[e] = vy[e];
+    }
+  };
+
+  // the largest exponent, the scale it calls for, and ||A||_F^2 in block order (volatile:
+  // written by other blocks of this launch)
+  int E = 0;
+#pragma unroll
+  for (int e = 0; e < EA; ++e) E = max(E, max(exponent_field(xs[e]), exponent_field(ys[e])));
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (lane == 0) atomicMax(a.top, E);
+  double al, be, ga, floor2 = 0.0, scale = 1.0;
+  dots(al, be, ga);
+  totals(true, al, be, ga);
+  if (tid == 0) a.part[k] = al + be;
+  int sweep = 0;
+  bool converged = false, ok = grid_barrier(a.bar);
+  if (ok) {
+    scale = range_scale(*const_cast<volatile int*>(a.top));
+    if (scale != 1.0) {  // the same in every block
+#pragma unroll
+      for (int e = 0; e < EA; ++e) {
+        xs[e] *= scale;
+        ys[e] *= scale;
+      }
+      dots(al, be, ga);
+      totals(true, al, be, ga);
+      if (tid == 0) a.part[K + k] = al + be;
+      ok = grid_barrier(a.bar);
+    }
+  }
+  if (ok) {
+    volatile const double* const part = a.part + (scale != 1.0 ? K : 0);
+    double f = 0.0;
+    for (int i = lane; i < K; i += 32) f += part[i];
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    floor2 = 7.9e-31 * f;
+  }
+  uint32_t tag = 0;  // rounds done so far; a column sent after round t carries t + 1
+  for (; ok && sweep < a.max_sweeps; ++sweep) {
+    bool any = false;
+    for (int r = 0; r < L; ++r, ++tag) {
+      const bool moved = tag != 0;
+      if (moved) {
+        const ulonglong2* const bp = slot(tag & 1, k, 0);
+        const ulonglong2* const bq = slot(tag & 1, k, 1);
+        uint64_t t0 = 0;
+        for (int spin = 0;; ++spin) {
+          bool got = true;
+#pragma unroll
+          for (int e = 0; e < EA; ++e) {
+            const int i = tid + 128 * e;
+            if (i < m) {
+              if (k != 0 && k != last) got = get_tagged(bp + i, tag, xs[e]) && got;
+              got = get_tagged(bq + i, tag, ys[e]) && got;
+            }
+          }
+          if (got) break;
+          if ((spin & 63) == 0) {
+            const uint64_t now = global_ns();
+            if (spin == 0) t0 = now;
+            if (now - t0 >= limit) atomicExch(a.bar + 2, 1u);
+            if (*abort_flag != 0u) { ok = false; break; }
+          }
+        }
+      }
+      dots(al, be, ga);
+      if (!totals(ok, al, be, ga)) { ok = false; break; }
+      double c = 1.0, sn = 0.0;
+      const bool doit = jacobi_rotation(al, be, ga, floor2, a.tol, c, sn);
+      any = any || doit;
+      if (doit) {
+#pragma unroll
+        for (int e = 0; e < EA; ++e)
+          if (32 * warp + 128 * e < m) {
+            const double x = xs[e], y = ys[e];
+            xs[e] = c * x - sn * y;
+            ys[e] = sn * x + c * y;
+          }
+      }
+      ulonglong2* const dp = k != 0 ? slot((tag + 1) & 1, p_to, p_slot) : nullptr;
+      ulonglong2* const dq = k != last ? slot((tag + 1) & 1, k + 1, 1) : nullptr;
+#pragma unroll
+      for (int e = 0; e < EA; ++e) {
+        const int i = tid + 128 * e;
+        if (i < m) {
+          if (k != 0) put_tagged(dp + i, xs[e], tag + 1);
+          if (k != last) put_tagged(dq + i, ys[e], tag + 1);
+        }
+      }
+      if (moved) {
+        const ulonglong2* const bp = slot(tag & 1, k, 0) + m;
+        const ulonglong2* const bq = slot(tag & 1, k, 1) + m;
+        uint64_t t0 = 0;
+        for (int spin = 0;; ++spin) {
+          bool got = true;
+#pragma unroll
+          for (int e = 0; e < EV; ++e) {
+            const int i = tv + 128 * e;
+            if (i < N) {
+              if (k != 0 && k != last) got = get_tagged(bp + i, tag, vx[e]) && got;
+              got = get_tagged(bq + i, tag, vy[e]) && got;
+            }
+          }
+          if (got) break;
+          if ((spin & 63) == 0) {
+            const uint64_t now = global_ns();
+            if (spin == 0) t0 = now;
+            if (now - t0 >= limit) atomicExch(a.bar + 2, 1u);
+            if (*abort_flag != 0u) { ok = false; break; }
+          }
+        }
+      }
+      if (doit) {
+#pragma unroll
+        for (int e = 0; e < EV; ++e)
+          if ((((32 * warp + 64) & 127) + 128 * e) < N) {
+            const double x = vx[e], y = vy[e];
+            vx[e] = c * x - sn * y;
+            vy[e] = sn * x + c * y;
+          }
+      }
+#pragma unroll
+      for (int e = 0; e < EV; ++e) {
+        const int i = tv + 128 * e;
+        if (i < N) {
+          if (k != 0) put_tagged(dp + m + i, vx[e], tag + 1);
+          if (k != last) put_tagged(dq + m + i, vy[e], tag + 1);
+        }
+      }
+      if (r + 1 == L) break;  // the last round of a converged sweep is where the columns stay
+      advance();
+    }
+    if (!__syncthreads_and(ok)) { ok = false; break; }
+    if (any && tid == 0) atomicExch(a.rot + sweep, 1);
+    if (!grid_barrier(a.bar)) { ok = false; break; }
+    if (*const_cast<volatile int*>(a.rot + sweep) == 0) { converged = true; break; }
+    ++tag;
+    advance();
+  }
+  // norms, descending ranks (ties by index) and outputs of the columns the block ended with
+  if (ok) {
+    if (tid < 2) {
+      sig_s[tid] = sqrt(tid == 0 ? al : be);
+      a.sig[tid == 0 ? p : q] = sig_s[tid];
+    }
+    ok = grid_barrier(a.bar);
+  }
+  if (!ok) {
+    if (tid == 0) atomicMax(a.status, 2);
+    return;
+  }
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int col = w == 0 ? p : q;
+    if (col >= n) continue;  // the padding column
+    const double sj = sig_s[w];
+    int rk = 0;
+    for (int i0 = 0; i0 < n; i0 += 128) {
+      const int i = i0 + tid;
+      const double si = i < n ? *const_cast<volatile const double*>(a.sig + i) : -1.0;
+      rk += __syncthreads_count(i < n && (si > sj || (si == sj && i < col)));
+    }
+    const double inv = 1.0 / sj;
+#pragma unroll
+    for (int e = 0; e < EA; ++e) {
+      const int i = tid + 128 * e;
+      if (i < m) a.U[int64_t(i) * n + rk] = sj > 0.0 ? div_by(w == 0 ? xs[e] : ys[e], sj, inv) : 0.0;
+    }
+#pragma unroll
+    for (int e = 0; e < EV; ++e) {
+      const int i = tv + 128 * e;
+      if (i < n) a.V[int64_t(i) * n + rk] = w == 0 ? vx[e] : vy[e];
+    }
+    if (tid == 0) a.S[rk] = scale != 1.0 ? sj / scale : sj;
+  }
+  if (k == 0 && tid == 0 && !converged) atomicMax(a.status, 1);
+}
+
 __global__ void sumsq_kernel(const double* x, int64_t n, double* out) {
   double acc = 0.0;
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n;
@@ -648,10 +1015,67 @@ __global__ void permute_rows_kernel(const double* Ux, const int* perm, int n, do
 }
 
 // The single-block Jacobi keeps the whole m x N column-major copy in shared memory
-// (at most 200 KB); it is used for narrow matrices (N < 32) that fit.  Everything else,
-// including N = 2 with a tall m, takes the multi-block kernels, which handle one column
-// pair as well.
+// (at most 200 KB); it is used for narrow matrices (N < 32) that fit.  Columns of up to
+// 1024 rows with N <= 256 fit the registers of jacobi_ring_kernel's blocks; everything else,
+// including N = 2 with a tall m, takes the kernels that leave the columns in L2.
 bool single_block_fits(int64_t m, int N) { return N < 32 && m * N * int64_t(sizeof(double)) <= 200 * 1024; }
+// N / 2 <= 128 blocks of 128 threads must be co-resident: at least one per SM is
+bool ring_fits(int64_t m, int N) { return N >= 32 && N <= 256 && m <= 1024 && N / 2 <= sm_count(); }
+
+constexpr int kJacobiSweeps = 60;
+
+void launch_jacobi_small(const double* A, int64_t m, int n, int N, double* U, double* S, double* V, double tol,
+                         int* status_dev, cudaStream_t s) {
+  const int G = m <= 16 ? 16 : 32, threads = int(cdiv(int64_t(N / 2) * G, 32)) * 32;
+  const size_t sm = size_t(m * N + N * N) * sizeof(double);
+  const int most = 200 * 1024 + 30 * 30 * int(sizeof(double));
+  if (G == 16) {
+    jacobi_small_kernel<16><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, float(tol), status_dev);
+  } else {
+    ensure_smem_attr(reinterpret_cast<const void*>(jacobi_small_kernel<32>), most);
+    jacobi_small_kernel<32><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, float(tol), status_dev);
+  }
+  TATRG_CUDA(cudaGetLastError());
+}
+
+template <int EA, int EV>
+void launch_ring(RingArgs& a, cudaStream_t s) {
+  void* args[] = {&a};
+  TATRG_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(jacobi_ring_kernel<EA, EV>), dim3(a.N / 2),
+                                         dim3(128), args, 0, s));
+}
+
+void launch_jacobi_ring(const double* A, int m, int n, int N, double* U, double* S, double* V, double tol,
+                        int* status_dev, cudaStream_t s) {
+  // workspace: the ring's slots, partial sums and norms, the sweeps' flags and the barrier
+  const size_t ring = size_t(2) * (N / 2) * 2 * (m + N) * sizeof(ulonglong2), sums = size_t(2) * N * sizeof(double),
+               flags = (kJacobiSweeps + 5) * sizeof(int);
+  DevBuf ws(ring + sums + flags, s);
+  TATRG_CUDA(cudaMemsetAsync(ws.d(), 0, ws.bytes(), s));  // tags and flags start at zero
+  TATRG_CUDA(cudaMemsetAsync(status_dev, 0, sizeof(int), s));
+  RingArgs a;
+  a.A = A;
+  a.m = m;
+  a.n = n;
+  a.N = N;
+  a.U = U;
+  a.S = S;
+  a.V = V;
+  a.ring = ws.as<ulonglong2>();
+  a.part = reinterpret_cast<double*>(ws.as<char>() + ring);
+  a.sig = a.part + N;
+  a.rot = reinterpret_cast<int*>(ws.as<char>() + ring + sums);
+  a.bar = reinterpret_cast<unsigned*>(a.rot + kJacobiSweeps);
+  a.top = a.rot + kJacobiSweeps + 4;
+  a.status = status_dev;
+  a.max_sweeps = kJacobiSweeps;
+  a.tol = float(tol);
+  // registers for the columns: (A, V) chunks of 128 rows
+  if (m <= 128) launch_ring<1, 1>(a, s);
+  else if (m <= 256) launch_ring<2, 2>(a, s);
+  else if (m <= 512) launch_ring<4, 2>(a, s);
+  else launch_ring<8, 2>(a, s);
+}
 }  // namespace
 
 int cholesky_max_n() { return kCholMaxN; }
@@ -688,18 +1112,23 @@ void jacobi_svd(const double* A, int64_t m, int n, double* U, double* S, double*
   check_extent(S, n - 1, sizeof(double), "jacobi S");
   check_extent(V, int64_t(n) * n - 1, sizeof(double), "jacobi V");
   const int N = n + (n & 1);
+  const double tol = std::max(1e-15, 2.220446049250313e-16 * std::sqrt(double(m)));
+  if (single_block_fits(m, N)) {
+    launch_jacobi_small(A, m, n, N, U, S, V, tol, status_dev, s);
+    if (st) st->launches += 1;
+    return;
+  }
+  if (ring_fits(m, N)) {
+    launch_jacobi_ring(A, int(m), n, N, U, S, V, tol, status_dev, s);
+    if (st) st->launches += 1;
+    return;
+  }
   DevBuf ac(size_t(m) * N * sizeof(double), s), vc(size_t(N) * N * sizeof(double), s);
   int64_t tot = m * N + int64_t(N) * N;
   to_colmajor_kernel<<<int(std::min<int64_t>(cdiv(tot, 256), 2048)), 256, 0, s>>>(A, m, n, N,
                                                                                   ac.d(), vc.d());
   TATRG_CUDA(cudaGetLastError());
-  const double tol = std::max(1e-15, 2.220446049250313e-16 * std::sqrt(double(m)));
-  if (single_block_fits(m, N)) {
-    int threads = 32 * std::max(1, std::min(32, N / 2));
-    ensure_smem_attr(reinterpret_cast<const void*>(jacobi_kernel), 200 * 1024);
-    jacobi_kernel<<<1, threads, size_t(m * N) * sizeof(double), s>>>(ac.d(), m, N, vc.d(), 60, tol, status_dev);
-    TATRG_CUDA(cudaGetLastError());
-  } else {
+  {
     // one block per column pair, all sweeps in one cooperative launch (its blocks are
     // co-resident by construction; the barrier between rounds gives up after 2 s and
     // reports status 2)
@@ -791,21 +1220,20 @@ void jacobi_svd_noalloc(const double* A, int64_t m, int n, double* U, double* S,
   double* fro2 = sig + 2 * N;
   int* rot = reinterpret_cast<int*>(fro2 + 1);
   int* status = reinterpret_cast<int*>(fro2 + 2);
-  int64_t tot = m * N + int64_t(N) * N;
-  to_colmajor_kernel<<<int(std::min<int64_t>(cdiv(tot, 256), 2048)), 256, 0, s>>>(A, m, n, N, ac, vc);
-  TATRG_CUDA(cudaGetLastError());
   const double tol = std::max(1e-15, 2.220446049250313e-16 * std::sqrt(double(m)));
-  int converged = 0;
   if (single_block_fits(m, N)) {
-    int threads = 32 * std::max(1, std::min(32, N / 2));
-    TATRG_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    jacobi_kernel<<<1, threads, size_t(m * N) * sizeof(double), s>>>(ac, m, N, vc, 60, tol, status);
-    TATRG_CUDA(cudaGetLastError());
+    launch_jacobi_small(A, m, n, N, U, S, V, tol, status, s);
     int h = 1;
     TATRG_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));
     TATRG_CUDA(cudaStreamSynchronize(s));
-    converged = (h == 0);
-  } else {
+    TATRG_CHECK(h == 0, TATRG_ENUMERIC, "svd_noalloc: Jacobi SVD did not converge");
+    return;
+  }
+  int64_t tot = m * N + int64_t(N) * N;
+  to_colmajor_kernel<<<int(std::min<int64_t>(cdiv(tot, 256), 2048)), 256, 0, s>>>(A, m, n, N, ac, vc);
+  TATRG_CUDA(cudaGetLastError());
+  int converged = 0;
+  {
     TATRG_CUDA(cudaMemsetAsync(fro2, 0, sizeof(double), s));
     sumsq_kernel<<<int(std::min<int64_t>(cdiv(m * N, 256), 1024)), 256, 0, s>>>(ac, m * N, fro2);
     TATRG_CUDA(cudaGetLastError());

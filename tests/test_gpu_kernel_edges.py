@@ -48,3 +48,58 @@ def test_fp64_contraction_permuted_modes(torch, K, L):
     want = np.einsum("kila,bljk->aibj", A, B)
     bound = (K * L + 4) * 2 * EPS * np.einsum("kila,bljk->aibj", np.abs(A), np.abs(B))
     assert np.all(np.abs(C.cpu().numpy() - want) <= bound)
+
+
+def _svd(torch, fn, A):
+    m, n = A.shape
+    U, S, V = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((m, n), (n,), (n, n)))
+    fn(_dev(torch, A), U, S, V)
+    torch.cuda.synchronize()
+    return U.cpu().numpy(), S.cpu().numpy(), V.cpu().numpy()
+
+
+@pytest.mark.parametrize("m,n", [
+    (2, 2), (3, 1), (16, 16), (16, 15), (17, 16), (17, 17), (30, 30), (31, 29), (800, 30), (12000, 2),
+    (32, 31), (32, 32), (40, 33), (128, 128), (129, 128), (144, 143), (256, 256), (257, 200), (512, 64),
+    (513, 40), (1024, 34), (1025, 33), (300, 258)])
+def test_svd_kernel_boundaries(torch, m, n):
+    """The one-block form (n < 32, lane groups of 16 and 32), the ring of register-held columns
+    (up to 256 columns, 1024 rows, in chunks of 128 rows) and the form for larger matrices.
+    A column meets n rotations a sweep and these matrices need at most 12 sweeps; a rotation
+    adds a relative error of about 6 eps to the columns (Higham, Sec. 19.6)."""
+    rng = np.random.default_rng(1000 * n + m)
+    A = rng.standard_normal((m, n)) * 0.97 ** np.arange(n)
+    u, s, v = _svd(torch, tg.svd, A)
+    tol = 72 * max(n, 2) * EPS
+    assert np.all(np.diff(s) <= 0)
+    assert np.linalg.norm((u * s) @ v.T - A) <= tol * np.linalg.norm(A)
+    assert np.max(np.abs(v.T @ v - np.eye(n))) <= tol
+    assert np.max(np.abs(u.T @ u - np.eye(n))) <= tol
+    assert np.max(np.abs(s - np.linalg.svd(A, compute_uv=False))) <= tol * s[0]
+
+
+@pytest.mark.parametrize("scale", [1e-150, 1e-70, 1e70, 1e150])
+@pytest.mark.parametrize("m,n", [(20, 12), (60, 40)])
+def test_svd_of_scaled_matrices(torch, m, n, scale):
+    """Entries far from 1: the rotation's float arithmetic works on scaled values, so a power
+    of ten only rescales the singular values."""
+    rng = np.random.default_rng(5)
+    A = rng.standard_normal((m, n)) * 0.5 ** np.arange(n)
+    u, s, v = _svd(torch, tg.svd, A * scale)
+    tol = 72 * n * EPS
+    assert np.allclose(s / scale, np.linalg.svd(A, compute_uv=False), rtol=tol * 100, atol=tol)
+    assert np.linalg.norm((u * (s / scale)) @ v.T - A) <= tol * np.linalg.norm(A)
+
+
+def test_svd_of_zero_and_repeated_columns(torch):
+    """Zero columns give zero singular values and zero columns of U; V stays orthonormal."""
+    rng = np.random.default_rng(6)
+    for m, n in ((20, 12), (70, 48)):
+        A = rng.standard_normal((m, n))
+        A[:, 3] = 0.0
+        A[:, 7] = A[:, 1]
+        u, s, v = _svd(torch, tg.svd, A)
+        tol = 72 * n * EPS
+        assert np.linalg.norm((u * s) @ v.T - A) <= tol * np.linalg.norm(A)
+        assert np.max(np.abs(v.T @ v - np.eye(n))) <= tol
+        assert np.all(s[n - 2:] <= tol * s[0])
