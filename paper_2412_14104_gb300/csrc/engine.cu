@@ -71,10 +71,7 @@ OrthResult Engine::cholqr2(const double* Y, int64_t m, int64_t n, double shift, 
   const double* src = Y;
   for (int pass = 0; pass < passes; ++pass) {
     mm(n, n, m, src, n, true, src, n, false, G.d(), n);
-    cholesky(G.d(), int(n), Rk.d(), flag(0), pass == 0 ? shift : 0.0, s_);
-    st_.launches++;
-    if (read_flag(0) != 0) { ok = false; return out; }
-    tri_inverse(Rk.d(), int(n), Ri.d(), s_);
+    cholesky_inverse(G.d(), int(n), Rk.d(), Ri.d(), flag(0), pass == 0, pass == 0 ? shift : 0.0, s_);
     st_.launches++;
     DMat nxt;
     nxt.buf = dalloc(m * n, s_);
@@ -90,7 +87,9 @@ OrthResult Engine::cholqr2(const double* Y, int64_t m, int64_t n, double shift, 
     cur = std::move(nxt);
     src = cur.p();
   }
-  ok = true;
+  // a breakdown in any pass: its factors are zero, and so is what the later passes made of them
+  ok = read_flag(0) == 0;
+  if (!ok) return out;
   out.Q = std::move(cur);
   out.R.buf = std::move(Racc);
   out.R.rows = n;
@@ -149,10 +148,7 @@ Engine::MetricOrth Engine::orth_metric(const double* X, int64_t nin, int64_t w, 
   for (int pass = 0; pass < passes; ++pass) {
     metric(cur.p(), w, U.p());
     mm(w, w, nin, cur.p(), w, true, U.p(), w, false, G.d(), w);
-    cholesky(G.d(), int(w), Rk.d(), flag(0), pass == 0 ? shift : 0.0, s_);
-    st_.launches++;
-    if (read_flag(0) != 0) return out;  // ok = false
-    tri_inverse(Rk.d(), int(w), Ri.d(), s_);
+    cholesky_inverse(G.d(), int(w), Rk.d(), Ri.d(), flag(0), pass == 0, pass == 0 ? shift : 0.0, s_);
     st_.launches++;
     DMat nxt;
     nxt.buf = dalloc(nin * w, s_);
@@ -167,6 +163,7 @@ Engine::MetricOrth Engine::orth_metric(const double* X, int64_t nin, int64_t w, 
     }
     cur = std::move(nxt);
   }
+  if (read_flag(0) != 0) return out;  // a breakdown in some pass: ok = false
   metric(cur.p(), w, U.p());  // U = G V for the final basis
   out.V = std::move(cur);
   out.U = std::move(U);

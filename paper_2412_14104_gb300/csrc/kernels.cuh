@@ -74,10 +74,11 @@ void check_finite(const double* x, int64_t n, int* bad_dev, cudaStream_t s);
 // linalg.cu ---------------------------------------------------------------------------
 // largest n of the one-block Cholesky (its working matrix lives in shared memory)
 int cholesky_max_n();
-// Cholesky G = R^T R of an n x n SPD matrix (row-major); R upper (row-major, zero below).
-// *status_dev = 0 on success, 1 when a pivot is not positive relative to its diagonal.
-void cholesky(const double* G, int n, double* R, int* status_dev, double shift_rel,
-              cudaStream_t s);
+// Cholesky G + shift_rel tr(G) I = R^T R of an n x n SPD matrix (row-major) and Rinv = R^-1;
+// R, Rinv upper (row-major, zero below).  *status_dev = 1 when a pivot is not positive
+// relative to its diagonal (R = Rinv = 0 then); otherwise 0 when `first`, else unchanged.
+void cholesky_inverse(const double* G, int n, double* R, double* Rinv, int* status_dev, bool first, double shift_rel,
+                      cudaStream_t s);
 // inverse of an upper-triangular n x n matrix (row-major)
 void tri_inverse(const double* R, int n, double* Rinv, cudaStream_t s);
 // One-sided Jacobi SVD of a row-major m x n (m >= n): U (m x n), S (n), V (n x n) with

@@ -1,8 +1,8 @@
-// Small dense FP64 linear algebra: Cholesky (the core of CholeskyQR2; one block), the
-// inverse of the triangular factor (one warp per column), and the one-sided (Hestenes)
-// Jacobi SVD used for every core SVD / PSD eigenproblem of the RG step (swap core, triad
-// Gram eigenvectors, squeezer factors and core, re-split): one block in shared memory for
-// small problems, otherwise one cooperative grid with a block per column pair.
+// Small dense FP64 linear algebra: Cholesky with the inverse of its factor (the core of
+// CholeskyQR2; one cluster), and the one-sided (Hestenes) Jacobi SVD used for every core SVD
+// / PSD eigenproblem of the RG step (swap core, triad Gram eigenvectors, squeezer factors
+// and core, re-split): one block in shared memory for small problems, otherwise one
+// cooperative grid with a block per column pair.
 
 #include <cooperative_groups.h>
 
@@ -14,68 +14,182 @@ namespace {
 
 constexpr int kCholMaxN = 168;
 
-// Right-looking Cholesky G + shift I = R^T R with the upper triangle of the working
-// matrix in shared memory (full n x n storage, n <= kCholMaxN: 168^2 doubles and the
-// kernel's own arrays fill the 227 KB a block may hold).  Step j scales row j by the
-// pivot square root, then subtracts the outer product of the scaled row from the trailing
-// block; the thread that updates the next diagonal entry takes its square root at once
-// (FP64 square roots and divisions are scarce on this GPU, so they are not repeated per
-// thread), which leaves two block barriers per step.  A pivot at or below 1e-14 of its
-// original diagonal entry is a breakdown (status 1).
-__global__ void __launch_bounds__(1024) cholesky_kernel(const double* G, int n, double* R,
-                                                        int* status, double shift_rel) {
-  extern __shared__ double W[];
-  __shared__ double shift, djj_s[2];
+// Cholesky G + shift I = R^T R and X = R^-1 in one launch: the row operations that turn the
+// upper triangle of G into R turn the identity beside it into R^-T, panel by panel of CB
+// rows, right-looking.  A cluster of CL blocks holds the 2 n columns in shared memory
+// (column c of either half in block c % CL).  Per panel:
+//   - warp 0 of every block reads the CB x CB diagonal block out of the others' shared memory
+//     and eliminates it in registers, a column a lane (lanes 0..15: R's rows, lanes 16..31:
+//     T = R_JJ^-T), every block the same numbers;
+//   - each block replaces the panel's rows of its own columns by T times them;
+//   - each block reads the panel's rows of R (the multipliers) out of the others' shared
+//     memory and updates its own columns below the panel, first the next diagonal block's:
+//     warp 0 goes on to that block while the other warps finish the update.
+//
+// What bounds it: the elimination's chain, per row a reciprocal and CB FP64 instructions of
+// 64 clocks (about 0.45 us a row), under which the update of n^3 / (3 CL) multiply-adds (1.7
+// a clock per SM) disappears.  One block alone took 174 us at n = 96, half of it the SM's FP64
+// rate, and the inverse after it 94 us (a warp a column, a division and a shuffled sum a
+// row); see launch_chol for this form.
+//
+// A pivot at or below 1e-14 of its original diagonal entry, or not finite, is a breakdown:
+// status 1 and R = X = 0.
+constexpr int CB = 16;
+
+template <int CL>
+__global__ void __launch_bounds__(256) chol_inverse_kernel(const double* G, int n, double* R, double* X, int* status,
+                                                           int first, double shift_rel) {
+  namespace cg = cooperative_groups;
+  extern __shared__ double sm[];
+  __shared__ double T[CB][CB + 1], Rd[CB][CB + 1];
+  __shared__ int64_t thr[kCholMaxN];  // bits of the smallest pivot that is no breakdown
+  __shared__ double red[8];
   __shared__ int fail_s;
-  __shared__ double red[32];
-  __shared__ double ref[kCholMaxN];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int tx = tid & 31, ty = tid >> 5;  // 32 x 32 threads over (k, i)
-  {
-    double tr = 0.0;
-    for (int i = tid; i < n; i += nt) tr += G[int64_t(i) * n + i];
-    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-    if (tx == 0) red[ty] = tr;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (nt >> 5); ++w) t += red[w];
-      shift = shift_rel * t;
-      fail_s = 0;
-    }
-    __syncthreads();
-  }
-  const double sh = shift;
-  for (int e = tid; e < n * n; e += nt) {
-    const int i = e / n, k = e - (e / n) * n;
-    W[e] = (k >= i) ? G[e] + (i == k ? sh : 0.0) : 0.0;
-    if (i == k) ref[i] = G[e] + sh;
-  }
-  __syncthreads();
-  // pivot j is checked and rooted by thread 0, which also updates entry (j, j) in step j - 1
-  auto pivot = [&](int j) {
-    const double d = W[j * n + j];
-    if (!(d > 1e-14 * ref[j]) || !(ref[j] > 0.0)) fail_s = 1;
-    else djj_s[j & 1] = sqrt(d);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = CL > 1 ? int(cg::this_cluster().block_rank()) : 0;
+  auto cluster_sync = [] {
+    if (CL > 1) cg::this_cluster().sync();
+    else __syncthreads();
   };
-  if (tid == 0) pivot(0);
-  for (int j = 0; j < n; ++j) {
-    __syncthreads();
-    if (fail_s) break;  // uniform across the block
-    const double djj = djj_s[j & 1];
-    for (int k = j + tid; k < n; k += nt) W[j * n + k] = (k == j) ? djj : W[j * n + k] / djj;
-    __syncthreads();
-    for (int i = j + 1 + ty; i < n; i += 32) {
-      const double a = W[j * n + i];
-      for (int k = i + ((tx - (i - (j + 1))) & 31); k < n; k += 32)
-        W[i * n + k] = fma(-a, W[j * n + k], W[i * n + k]);
+  const int ld = n | 1, nl = (n + CL - 1) / CL;
+  double* const Lc = sm;            // columns of the left half
+  double* const Rc = Lc + nl * ld;  // columns of the right half
+  double* const Mp = Rc + nl * ld;  // the panel's multipliers, row i at i (CB + 1)
+  // column c of the left half, wherever it is
+  auto left = [&](int c) -> const double* {
+    if (CL == 1) return Lc + c * ld;
+    return cg::this_cluster().map_shared_rank(Lc, c % CL) + (c / CL) * ld;
+  };
+  double tr = 0.0;
+  for (int i = tid; i < n; i += 256) tr += G[int64_t(i) * n + i];
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  if (lane == 0) red[warp] = tr;
+  if (tid == 0) fail_s = 0;
+  __syncthreads();
+  tr = 0.0;
+  for (int w = 0; w < 8; ++w) tr += red[w];
+  const double sh = shift_rel * tr;
+  for (int e = tid; e < nl * n; e += 256) {
+    const int i = e / nl, l = e - (e / nl) * nl, c = l * CL + rank;
+    if (c < n) {
+      Lc[l * ld + i] = i <= c ? G[int64_t(i) * n + c] + (i == c ? sh : 0.0) : 0.0;
+      Rc[l * ld + i] = i == c ? 1.0 : 0.0;
     }
-    if (tid == 0 && j + 1 < n) pivot(j + 1);  // thread 0 updated entry (j + 1, j + 1) above
+  }
+  for (int i = tid; i < n; i += 256) {
+    const double ref = G[int64_t(i) * n + i] + sh;
+    thr[i] = ref > 0.0 ? __double_as_longlong(1e-14 * ref) : 0x7FF0000000000000ll;
+  }
+  cluster_sync();
+
+  // the diagonal block from row j0 on, by warp 0
+  auto factor = [&](int j0) {
+    const int bs = min(CB, n - j0), k = lane & (CB - 1);
+    const bool lhs = lane < CB;
+    double col[CB];
+    const double* const src = (lhs && k < bs) ? left(j0 + k) + j0 : nullptr;
+#pragma unroll
+    for (int i = 0; i < CB; ++i) col[i] = (src && i <= k) ? src[i] : (i == k ? 1.0 : 0.0);
+    bool bad = false;
+    double dk = 1.0;  // lane k: pivot k
+    for (int j = 0; j < bs; ++j) {  // col[0] is the pivot row; the others move up as they are updated
+      const double row = col[0], d = __shfl_sync(0xffffffffu, row, j);
+      const int ex = exponent_field(d);
+      if (!(__double_as_longlong(d) > thr[j0 + j]) || ex == 0 || ex >= 2044) bad = true;
+      if (k == j) dk = d;
+      (lhs ? Rd[j] : T[j])[k] = row;
+      const double g = row * fast_rcp(bad ? 1.0 : d);
+#pragma unroll
+      for (int i = 1; i < CB; ++i)
+        if (i < bs - j) col[i - 1] = fma(-__shfl_sync(0xffffffffu, row, j + i), g, col[i]);
+    }
+    if (bad) dk = 1.0;
+    const double rs = fast_rsqrt(dk);
+    double sq = dk * rs;
+    sq = fma(0.5 * fma(-sq, sq, dk), rs, sq);  // sqrt(d)
+    for (int j = 0; j < bs; ++j) {
+      const double rj = __shfl_sync(0xffffffffu, rs, j);
+      double* const x = &(lhs ? Rd[j] : T[j])[k];
+      const double v = (lhs && k == j) ? sq : *x * rj;
+      *x = (lhs ? k >= j : k <= j) ? v : 0.0;
+    }
+    if (bad && lane == 0) fail_s = 1;
+  };
+  // rows of column c (a pointer to its storage) from i0 to i1 updated by the panel at j0
+  auto update = [&](double* col, int j0, int i0, int i1) {
+    for (int i = i0 + lane; i - lane < i1; i += 32) {
+      if (i < i1) {
+        double v = col[i];
+#pragma unroll
+        for (int l = 0; l < CB; ++l) v = fma(-Mp[i * (CB + 1) + l], col[j0 + l], v);
+        col[i] = v;
+      }
+    }
+  };
+
+  if (warp == 0) factor(0);
+  bool fail = false;
+  for (int j0 = 0; j0 < n; j0 += CB) {
+    const int bs = min(CB, n - j0), j1 = j0 + bs;
+    __syncthreads();
+    fail = fail_s != 0;
+    if (fail) break;  // every block eliminated the same numbers
+    // the panel's rows of the block's columns: T W (rows of W below T's diagonal only)
+    for (int e = tid; e < 2 * nl * CB; e += 256) {
+      const int row = e & (CB - 1), it = e / CB, half = it >= nl, l = half ? it - nl : it;
+      const int c = l * CL + rank;
+      double* const w = (half ? Rc : Lc) + l * ld + j0;
+      const bool on = c < n && row < bs && (half ? c < j0 : c >= j1);
+      double v = 0.0;
+      if (on)
+        for (int t = 0; t <= row; ++t) v = fma(T[row][t], w[t], v);
+      __syncwarp();
+      if (on) w[row] = v;
+      if (half && c >= j0 && c < j1 && row < bs) w[row] = T[row][c - j0];
+    }
+    cluster_sync();
+    // the diagonal block's own rows: the other blocks have read the old ones
+    for (int e = tid; e < nl * CB; e += 256) {
+      const int row = e & (CB - 1), l = e / CB, c = l * CL + rank;
+      if (c >= j0 && c < j1 && row < bs) Lc[l * ld + j0 + row] = Rd[row][c - j0];
+    }
+    if (j1 >= n) break;
+    for (int e = tid; e < (n - j1) * CB; e += 256) {
+      const int l = e & (CB - 1), i = j1 + e / CB;
+      Mp[i * (CB + 1) + l] = left(i)[j0 + l];
+    }
+    __syncthreads();
+    // the next diagonal block's columns first; then warp 0 eliminates that block beside the rest
+    const int j2 = min(n, j1 + CB);
+    for (int l = warp; l < nl; l += 8) {
+      const int c = l * CL + rank;
+      if (c >= j1 && c < j2) update(Lc + l * ld, j0, j1, c + 1);
+    }
+    cluster_sync();
+    if (warp == 0) {
+      factor(j1);
+    } else {
+      for (int it = warp - 1; it < 2 * nl; it += 7) {
+        const bool half = it >= nl;
+        const int l = half ? it - nl : it, c = l * CL + rank;
+        if (c >= n) continue;
+        if (half) {
+          if (c < j1) update(Rc + l * ld, j0, j1, n);
+        } else if (c >= j2) {
+          update(Lc + l * ld, j0, j1, c + 1);
+        }
+      }
+    }
   }
   __syncthreads();
-  const int fail = fail_s;
-  for (int e = tid; e < n * n; e += nt) R[e] = fail ? 0.0 : W[e];
-  if (tid == 0) *status = fail;
+  for (int e = tid; e < nl * n; e += 256) {
+    const int l = e / n, i = e - (e / n) * n, c = l * CL + rank;
+    if (c >= n) continue;
+    R[int64_t(i) * n + c] = (fail || i > c) ? 0.0 : Lc[l * ld + i];
+    X[int64_t(c) * n + i] = (fail || i < c) ? 0.0 : Rc[l * ld + i];
+  }
+  if (rank == 0 && tid == 0 && (first || fail)) *status = fail ? 1 : 0;
+  cluster_sync();  // no block leaves while another may still read its shared memory
 }
 
 // Inverse of an upper-triangular matrix: column c of X = R^-1 is the back substitution
@@ -1080,15 +1194,41 @@ void launch_jacobi_ring(const double* A, int m, int n, int N, double* U, double*
 
 int cholesky_max_n() { return kCholMaxN; }
 
-void cholesky(const double* G, int n, double* R, int* status_dev, double shift_rel,
-              cudaStream_t s) {
+namespace {
+// Cluster size by the update's share: n^3 / (3 CL) multiply-adds at 1.7 a clock stay below
+// the chain of n rows at ~900 clocks.
+template <int CL>
+void launch_chol(const double* G, int n, double* R, double* Rinv, int* status_dev, bool first, double shift_rel,
+                 cudaStream_t s) {
+  const int ld = n | 1, nl = (n + CL - 1) / CL;
+  const size_t sm = (size_t(2) * nl * ld + size_t(n) * (CB + 1)) * sizeof(double);
+  ensure_smem_attr(reinterpret_cast<const void*>(chol_inverse_kernel<CL>), int(sm));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  TATRG_CUDA(cudaLaunchKernelEx(&cfg, chol_inverse_kernel<CL>, G, n, R, Rinv, status_dev, first ? 1 : 0, shift_rel));
+  TATRG_CUDA(cudaGetLastError());
+}
+}  // namespace
+
+void cholesky_inverse(const double* G, int n, double* R, double* Rinv, int* status_dev, bool first, double shift_rel,
+                      cudaStream_t s) {
   check_extent(G, int64_t(n) * n - 1, sizeof(double), "cholesky input");
   check_extent(R, int64_t(n) * n - 1, sizeof(double), "cholesky output");
+  check_extent(Rinv, int64_t(n) * n - 1, sizeof(double), "cholesky inverse");
   TATRG_CHECK(n >= 1 && n <= kCholMaxN, TATRG_EINVAL, "cholesky: n must be <= 168");
-  const size_t sm = size_t(n) * n * sizeof(double);
-  ensure_smem_attr(reinterpret_cast<const void*>(cholesky_kernel), kCholMaxN * kCholMaxN * 8);
-  cholesky_kernel<<<1, 1024, sm, s>>>(G, n, R, status_dev, shift_rel);
-  TATRG_CUDA(cudaGetLastError());
+  if (n <= 32) launch_chol<1>(G, n, R, Rinv, status_dev, first, shift_rel, s);
+  else if (n <= 64) launch_chol<4>(G, n, R, Rinv, status_dev, first, shift_rel, s);
+  else launch_chol<8>(G, n, R, Rinv, status_dev, first, shift_rel, s);
 }
 
 void tri_inverse(const double* R, int n, double* Rinv, cudaStream_t s) {

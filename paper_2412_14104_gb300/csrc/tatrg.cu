@@ -1842,6 +1842,7 @@ tatrg_status tatrg_svd(int64_t m, int64_t n, const double* A, double* U, double*
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Engine e(s);
     SvdResult r = e.svd(A, m, n);
+    // a failed factorisation leaves the caller's arrays as they were
     TATRG_CUDA(cudaMemcpyAsync(U, r.U.p(), m * n * sizeof(double), cudaMemcpyDeviceToDevice, s));
     TATRG_CUDA(cudaMemcpyAsync(S, r.S.d(), n * sizeof(double), cudaMemcpyDeviceToDevice, s));
     TATRG_CUDA(cudaMemcpyAsync(V, r.V.p(), n * n * sizeof(double), cudaMemcpyDeviceToDevice, s));

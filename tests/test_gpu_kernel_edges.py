@@ -103,3 +103,35 @@ def test_svd_of_zero_and_repeated_columns(torch):
         assert np.linalg.norm((u * s) @ v.T - A) <= tol * np.linalg.norm(A)
         assert np.max(np.abs(v.T @ v - np.eye(n))) <= tol
         assert np.all(s[n - 2:] <= tol * s[0])
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 31, 32, 33, 48, 49, 64, 65, 95, 96, 128, 129, 144, 160, 167, 168])
+def test_cholesky_qr_panel_boundaries(torch, n):
+    """Orthonormalisation at the edges of the 16-row panels and of the cluster sizes.
+    CholeskyQR2: |Q^T Q - 1| <= 6 (m n + n (n + 1)) eps, |Q R - Y| <= 5 n^2 sqrt(n) eps |Y|
+    (Yamamoto et al. 2015, Theorems 3.2 and 3.3); R has a positive diagonal."""
+    m = 3 * n + 50
+    rng = np.random.default_rng(n)
+    Y = rng.standard_normal((m, n)) * 0.99 ** np.arange(n)
+    Q = torch.empty((m, n), dtype=torch.float64, device="cuda")
+    R = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    assert tg.orth(_dev(torch, Y), Q, R) == n
+    q, r = Q.cpu().numpy(), R.cpu().numpy()
+    assert np.array_equal(r, np.triu(r)) and np.all(np.diag(r) > 0)
+    assert np.linalg.norm(q.T @ q - np.eye(n), 2) <= 6 * (m * n + n * (n + 1)) * EPS
+    assert np.linalg.norm(q @ r - Y, 2) <= (5 * n * n * np.sqrt(n) + 20) * EPS * np.linalg.norm(Y, 2)
+
+
+@pytest.mark.parametrize("n,j", [(12, 0), (12, 11), (40, 16), (96, 95), (144, 100)])
+def test_cholesky_breakdown_in_any_panel(torch, n, j):
+    """A zero column makes pivot j exactly zero: the rank-revealing fallback returns n - 1 columns."""
+    rng = np.random.default_rng(n + j)
+    Y = rng.standard_normal((200, n))
+    Y[:, j] = 0.0
+    Q = torch.empty((200, n), dtype=torch.float64, device="cuda")
+    R = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    k = tg.orth(_dev(torch, Y), Q, R)
+    assert k == n - 1
+    q = Q.cpu().numpy().ravel()[:200 * k].reshape(200, k)
+    r = R.cpu().numpy().ravel()[:k * n].reshape(k, n)
+    assert np.linalg.norm(q @ r - Y) <= 72 * n * EPS * np.linalg.norm(Y)
