@@ -2,8 +2,15 @@
 // FP64 instruction holds a warp for 64 clocks whatever its active lanes; the library's
 // sqrt, division and 1/sqrt are dependent sequences of them (measured: 680, 420 and 370
 // clocks).  These take a float seed from the MUFU unit, with the exponents handled on the
-// integer pipe, and one third-order step in float64: 3 to 6 FP64 instructions, results
-// within about two units in the last place.  Arguments must be positive and normal.
+// integer pipe, and Newton steps in float64.  Arguments must be positive and normal.
+//
+// Two families: fast_* (3 to 5 instructions, results within about two units in the last
+// place) and near_* (4 to 6), whose last step corrects the result by its exact residual
+// (Markstein, IBM J. Res. Dev. 34, 1990): the correctly rounded value unless the exact one
+// lies within about 2^-80 of a rounding boundary.  The small factorisations use near_*, in
+// the operation order of the textbook formulas: the directions at the rounding floor of the
+// step's Grams are made of rounding errors, and a run depends on them at up to 1e-9 (chi = 8
+// sweeps), so a rounding changed here is a visible change of the results there.
 #pragma once
 
 #include <stdint.h>
@@ -52,21 +59,77 @@ __device__ __forceinline__ double fast_rsqrt(double d) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// r = 1 / (2 sqrt(d)) to ~1e-14, and sqrt(d) rounded (Goldschmidt's coupled iteration, then the
+// residual d - g^2)
+__device__ __forceinline__ double near_sqrt(double d, double& r) {
+  const int E = exponent_field(d), odd = (E & 1) ^ 1;
+  const float y = rsqrtf(d2f_scaled(d, E - odd));
+  const int sh = (1023 - (E - odd)) / 2;
+  double h = f2d_shift(y, sh - 1), g = d * f2d_shift(y, sh);
+  const double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  r = h;
+  return fma(fma(-g, g, d), h, g);
+}
+// 1 / d rounded, d of either sign, from r = 1 / d to ~1e-14
+__device__ __forceinline__ double near_rcp_from(double d, double r) { return fma(r, fma(-d, r, 1.0), r); }
+// the same for d a few units below a power of two (the pivots of a nearly orthonormal panel),
+// whose reciprocal lies within 2^-105 of a rounding boundary: a second step, and the one
+// mantissa that no number of steps rounds correctly, all ones, whose reciprocal is the power
+// of two's successor (Markstein)
+__device__ __forceinline__ double near_rcp_pivot(double d, double r) {
+  r = near_rcp_from(d, near_rcp_from(d, r));
+  constexpr uint64_t ones = 0xFFFFFFFFFFFFFull;
+  if ((uint64_t(__double_as_longlong(d)) & ones) == ones)
+    r = __longlong_as_double(int64_t((uint64_t(__double_as_longlong(r)) & ~ones) | 1ull));
+  return r;
+}
+// r = 1 / d to ~1e-14, d of either sign
+__device__ __forceinline__ double rcp14(double d) {
+  const int E = exponent_field(d);
+  const double y = f2d_shift(__frcp_rn(d2f_scaled(d, E)), 1023 - E);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+// x / d rounded, from r = 1 / d to ~1e-14
+__device__ __forceinline__ double near_div(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-q, d, x), r, q);
+}
+
 // Rotation of a pair of columns with squared norms al, be and inner product ga: the angle
 // t = tan of the smaller rotation that makes them orthogonal, c = 1 / sqrt(1 + t^2) and
 // s = c t.  No rotation (false) when a column lies at or below the floor or the inner
 // product is within tol of orthogonal.  The test and the first estimate of t are float
 // arithmetic on values scaled by the larger norm's exponent; one Newton step in float64
 // takes t to ~1e-14 and c, s to rounding: 11 FP64 instructions.
-__device__ __forceinline__ bool jacobi_rotation(double al, double be, double ga, double floor2, float tol,
+// EXACT: t, c and s by the textbook formulas with every operation correctly rounded (near_*,
+// 28 FP64 instructions).
+template <bool EXACT>
+__device__ __forceinline__ bool jacobi_rotation(double al, double be, double ga, double floor2, double tol,
                                                 double& c, double& s) {
   // non-negative doubles compare as integers
   const int64_t fl = __double_as_longlong(floor2), ia = __double_as_longlong(al), ib = __double_as_longlong(be);
   const int E = int(uint64_t(ia > ib ? ia : ib) >> 52);
   if (!(ia > fl && ib > fl) || E >= 0x7FF) return false;
   const float gf = d2f_scaled(ga, E), ag = fabsf(gf);
-  if (!(ag > tol * sqrtf(d2f_scaled(al, E) * d2f_scaled(be, E)))) return false;
+  const float bound = float(tol) * sqrtf(d2f_scaled(al, E) * d2f_scaled(be, E));
+  if (EXACT && fabsf(ag - bound) < 1e-5f * bound) {  // too close for float
+    if (!(fabs(ga) > tol * sqrt(al) * sqrt(be))) return false;
+  } else if (!(ag > bound)) {
+    return false;
+  }
   const double d = be - al;
+  if (EXACT) {
+    const double g2 = 2.0 * ga, zeta = near_div(d, g2, rcp14(g2));
+    double h;
+    const double den = fabs(zeta) + near_sqrt(fma(zeta, zeta, 1.0), h);
+    const double t = copysign(near_rcp_from(den, rcp14(den)), zeta);
+    const double root = near_sqrt(fma(t, t, 1.0), h);
+    c = near_rcp_from(root, 2.0 * h);
+    s = c * t;
+    return true;
+  }
   const float df = d2f_scaled(d, E), h = 0.5f * df, ah = fabsf(h);
   const float hi = fmaxf(ah, ag), q = fminf(ah, ag) / hi;
   const float tf = gf / (h + copysignf(hi * sqrtf(fmaf(q, q, 1.0f)), h));

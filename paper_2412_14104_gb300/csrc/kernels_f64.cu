@@ -15,9 +15,10 @@ namespace tatrg {
 // scheduling.
 //
 // What bounds it is the FP64 pipe: about two fused multiply-adds a clock per SM, padding
-// included, so one 64 x 64 x 16 tile holds an SM for 16 us.  gemm_plan picks the tile and
-// the split by that cost: large outputs keep T = 64 (2.1e9 flop in 1.8 ms, 1.18 of the
-// 1.25 TFLOP/s peak), the contractions of small bonds take smaller tiles on more SMs.
+// included, so one 64 x 64 x 16 tile holds an SM for 16 us.  gemm_tile picks the tile by
+// that cost: large outputs take whichever fills the last round best (2.1e9 flop in 1.75 ms,
+// 1.23 of the 1.25 TFLOP/s peak; 1.82 ms with 64 x 64 alone), the contractions of small
+// bonds take smaller tiles on more SMs (36 us down to 6 in a chi = 6 run).
 namespace {
 constexpr int BK = 16;
 constexpr int KTAB = 256;  // K offsets decomposed at a time, one per thread
@@ -196,32 +197,29 @@ __global__ void scale_modes_kernel(double* C, DevModes m, DevModes n, int64_t M,
   }
 }
 
-// Tile and K split of a contraction, by modelled time in clocks.  A T x T tile costs
-// 8 T^2 clocks per K tile of 16 on the FP64 pipe (two fused multiply-adds a clock), and at
-// least the latency of its loads and barriers; blocks on one SM share the pipe, so the
-// launch takes as many rounds as the fullest SM has blocks.  A split adds the launch of
-// the second kernel and its pass over the partials.
-struct GemmPlan {
-  int tile, split;
-};
+// K split of a contraction: enough 64 x 64 tiles and K ranges for four blocks per SM, ranges
+// of at least 64 elements.  It fixes the order of summation, so it does not depend on the
+// tile: a contraction gives the same bits whatever tile computes it.
+int gemm_split(int64_t M, int64_t N, int64_t K) {
+  const int64_t tiles = cdiv(M, 64) * cdiv(N, 64), target = 4 * int64_t(sm_count());
+  if (tiles >= target || K <= 4 * BK) return 1;
+  return int(std::min<int64_t>(std::min<int64_t>(cdiv(target, tiles), cdiv(K, 4 * BK)), 1024));
+}
 
-GemmPlan gemm_plan(int64_t M, int64_t N, int64_t K) {
-  const int64_t sms = sm_count(), ktiles = cdiv(K, BK);
-  GemmPlan best{64, 1};
+// Tile of a contraction cut into `split` K ranges, by modelled time: a T x T tile costs 8 T^2
+// clocks per K tile of 16 on the FP64 pipe (two fused multiply-adds a clock), and at least
+// the latency of its loads and barriers; blocks on one SM share the pipe, so the launch takes
+// as many rounds as the fullest SM has blocks.  Ties go to the larger tile (fewer loads).
+int gemm_tile(int64_t M, int64_t N, int split) {
+  const int64_t sms = sm_count();
+  int best = 64;
   double best_t = 0.0;
   for (int T : {64, 32, 16}) {
-    const int64_t tiles = cdiv(M, T) * cdiv(N, T);
     if (T < 64 && cdiv(std::min(M, N), T) > 65535) break;  // grid.y: the shorter side
-    const double step = std::max(8.0 * T * T, 1000.0);
-    for (int64_t want = 1; want <= 1024 && want <= std::max<int64_t>(1, ktiles / 2); want *= 2) {
-      const int64_t per = cdiv(ktiles, want), split = cdiv(ktiles, std::max<int64_t>(per, 1));
-      double t = double(cdiv(tiles * std::max<int64_t>(split, 1), sms)) * double(per) * step;
-      if (split > 1) t += 6000.0 + double(M) * double(N) * double(split) / (2.0 * double(sms));
-      if (best_t == 0.0 || t < 0.97 * best_t) {
-        best_t = t;
-        best = GemmPlan{T, int(want)};
-      }
-      if (tiles * want >= 8 * sms) break;  // more splits only add partials
+    const double t = double(cdiv(cdiv(M, T) * cdiv(N, T) * split, sms)) * std::max(8.0 * T * T, 1000.0);
+    if (best_t == 0.0 || t < 0.97 * best_t) {
+      best_t = t;
+      best = T;
     }
   }
   return best;
@@ -261,8 +259,7 @@ void gemm_f64(const GemmDesc& d0, const double* A, const double* B, double* C, c
   g.C = C;
   g.a_mcontig = stride1_first(d.m, true) && !stride1_first(d.k, true);
   g.b_ncontig = stride1_first(d.n, true) && !stride1_first(d.k, false);
-  const GemmPlan plan = gemm_plan(M, N, K);
-  int split = plan.split;
+  int split = gemm_split(M, N, K);
   int64_t kchunk = cdiv(cdiv(K, split), BK) * BK;
   split = int(cdiv(K, kchunk));
   if (K == 0) { split = 1; kchunk = 0; }
@@ -284,7 +281,7 @@ void gemm_f64(const GemmDesc& d0, const double* A, const double* B, double* C, c
     work.alloc(size_t(split) * size_t(M) * size_t(N) * sizeof(double), s);
     g.W = work.d();
   }
-  const int T = plan.tile;
+  const int T = gemm_tile(M, N, split);
   dim3 grid(unsigned(cdiv(M, T)), unsigned(cdiv(N, T)), unsigned(split));
   TATRG_CHECK(cdiv(N, T) <= 65535 && cdiv(M, T) < (int64_t(1) << 31), TATRG_EINVAL,
               "gemm_f64: problem too large for the grid");

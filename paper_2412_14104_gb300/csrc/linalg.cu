@@ -46,18 +46,14 @@ __global__ void __launch_bounds__(256) chol_inverse_kernel(const double* G, int 
   __shared__ double red[8];
   __shared__ int fail_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rank = CL > 1 ? int(cg::this_cluster().block_rank()) : 0;
-  auto cluster_sync = [] {
-    if (CL > 1) cg::this_cluster().sync();
-    else __syncthreads();
-  };
+  const int rank = int(cg::this_cluster().block_rank());
+  auto cluster_sync = [] { cg::this_cluster().sync(); };
   const int ld = n | 1, nl = (n + CL - 1) / CL;
   double* const Lc = sm;            // columns of the left half
   double* const Rc = Lc + nl * ld;  // columns of the right half
   double* const Mp = Rc + nl * ld;  // the panel's multipliers, row i at i (CB + 1)
   // column c of the left half, wherever it is
   auto left = [&](int c) -> const double* {
-    if (CL == 1) return Lc + c * ld;
     return cg::this_cluster().map_shared_rank(Lc, c % CL) + (c / CL) * ld;
   };
   double tr = 0.0;
@@ -192,6 +188,101 @@ __global__ void __launch_bounds__(256) chol_inverse_kernel(const double* G, int 
   cluster_sync();  // no block leaves while another may still read its shared memory
 }
 
+// The same for n <= 32, one block of four warps, lane = column.  Warp w holds rows w, w + 4, ...
+// of the working matrix in registers; step j: row j's warp takes the root of the pivot and
+// divides its row, all warps subtract its multiples from their rows.  The inverse follows
+// by back substitution of all columns at once: row i of X is ((i == c) - sum_k R_ik X_kc) /
+// R_ii, each warp summing every fourth term, in the order of a 32-lane butterfly.  Operations
+// and their order are those of a textbook Cholesky and substitution (near_*: see there).
+//
+// Bound by two FP64 chains of about 1000 and 750 clocks a row: 11 us at n = 12, where one
+// block of 1024 threads and a warp per column of the inverse took 18 + 12 us and a host read
+// of the status between them.
+__global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G, int n, double* R, double* X,
+                                                                 int* status, int first, double shift_rel) {
+  __shared__ double Rs[32][33], Xs[32][33], part[2][4][32], inv[32];
+  __shared__ int64_t thr[32];
+  __shared__ int fail_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double tr = lane < n ? G[lane * n + lane] : 0.0;
+  const double gd = tr;
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  const double sh = shift_rel * tr, ref = gd + sh;
+  if (warp == 0) {
+    thr[lane] = ref > 0.0 ? __double_as_longlong(1e-14 * ref) : 0x7FF0000000000000ll;
+    if (lane == 0) fail_s = 0;
+  }
+  double v[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = 4 * u + warp;
+    v[u] = (i < n && lane >= i && lane < n) ? G[i * n + lane] + (i == lane ? sh : 0.0) : 0.0;
+    Rs[i][lane] = 0.0;
+    Xs[i][lane] = 0.0;
+  }
+  __syncthreads();
+  bool fail = false;
+  for (int j0 = 0; j0 < n && !fail; j0 += 4) {  // v[u] is row j0 + 4 u + warp
+    for (int w = 0; w < 4 && j0 + w < n; ++w) {
+      const int j = j0 + w;
+      if (warp == w) {
+        const double d = __shfl_sync(0xffffffffu, v[0], j);
+        const int ex = exponent_field(d);
+        const bool bad = !(__double_as_longlong(d) > thr[j]) || ex == 0 || ex >= 2044;
+        double h;
+        const double root = near_sqrt(bad ? 1.0 : d, h), r = near_rcp_pivot(root, 2.0 * h);
+        if (lane >= j) Rs[j][lane] = lane == j ? root : near_div(v[0], root, r);
+        if (lane == j) {
+          inv[j] = r;
+          if (bad) fail_s = 1;
+        }
+      }
+      __syncthreads();
+      fail = fail_s != 0;
+      if (fail) break;
+      const double g = Rs[j][lane];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = j0 + 4 * u + warp;
+        if (i > j && i < n) v[u] = fma(-Rs[j][i], g, v[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 7; ++u) v[u] = v[u + 1];
+  }
+  if (!fail) {
+    for (int i = n - 1; i >= 0; --i) {
+      const int cnt = n - 1 - i;  // terms k = i + 1 + l, l < cnt; this warp's are l = 4 t + warp
+      double pr[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int l = 4 * t + warp;
+        pr[t] = 0.0;
+        if (l < cnt) pr[t] = __dmul_rn(Rs[i][i + 1 + l], Xs[i + 1 + l][lane]);  // not fused into the sum
+      }
+      // lanes l and l + 16, then + 8, then + 4 of the butterfly; absent terms are zeros
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int t = 0; t < o; ++t)
+          if (4 * (t + o) + warp < cnt) pr[t] += pr[t + o];
+      part[i & 1][warp][lane] = pr[0];
+      __syncthreads();
+      const double acc = (part[i & 1][0][lane] + part[i & 1][2][lane]) + (part[i & 1][1][lane] + part[i & 1][3][lane]);
+      // every warp forms and writes the same row: none waits for another's
+      Xs[i][lane] = i == lane ? inv[i] : near_div(0.0 - acc, Rs[i][i], inv[i]);
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < n * n; e += 128) {
+    const int i = e / n, c = e - (e / n) * n;
+    R[e] = fail ? 0.0 : Rs[i][c];
+    X[e] = (fail || i > c) ? 0.0 : Xs[i][c];
+  }
+  if (tid == 0 && (first || fail)) *status = fail ? 1 : 0;
+}
+
 // Inverse of an upper-triangular matrix: column c of X = R^-1 is the back substitution
 // R x = e_c, independent of the other columns, so one warp solves one column (x in the
 // warp's slice of shared memory, the inner products split across lanes); no block-wide
@@ -260,7 +351,7 @@ __device__ __forceinline__ double div_by(double x, double y, double r) {
 // one block, the columns of A and V in shared memory, the whole factorisation in one launch
 // (transposed load, sweeps, column norms, descending order, scaled output).
 //
-// Bound by FP64 latency: a round is a chain of about 30 FP64 instructions of 64 clocks
+// Bound by FP64 latency: a round is a chain of about 45 FP64 instructions of 64 clocks
 // (inner products, their reduction, the rotation's scalars, the update).  So a column pair
 // has one group of G lanes (16 for m <= 16, which packs two pairs into a warp), the groups
 // of a round spread over the SM's four FP64 ports, the reduction is group_sum3 and the
@@ -272,7 +363,7 @@ __device__ __forceinline__ double div_by(double x, double y, double r) {
 // inner product above tol forever.
 template <int G>
 __global__ void __launch_bounds__(512) jacobi_small_kernel(const double* A, int64_t m, int n, int N, double* U,
-                                                           double* S, double* V, int max_sweeps, float tol,
+                                                           double* S, double* V, int max_sweeps, double tol,
                                                            int* status) {
   extern __shared__ double Ac[];  // m x N, then V: N x N, both column-major
   __shared__ double wsum[16], sig[32], inv[32];
@@ -327,7 +418,7 @@ __global__ void __launch_bounds__(512) jacobi_small_kernel(const double* A, int6
         }
       }
       group_sum3<G>(al, be, ga);
-      if (active && jacobi_rotation(al, be, ga, floor2, tol, c, sn)) {
+      if (active && jacobi_rotation<true>(al, be, ga, floor2, tol, c, sn)) {
         for (int64_t i = g; i < m; i += G) {
           const double x = ap[i], y = aq[i];
           ap[i] = c * x - sn * y;
@@ -348,15 +439,20 @@ __global__ void __launch_bounds__(512) jacobi_small_kernel(const double* A, int6
   }
   // column norms by the same groups (columns 2k, 2k + 1), ranks (ties by index), outputs
   {
-    double a2 = 0.0, b2 = 0.0, z = 0.0;
-    if (active) {
-      const double* const ap = Ac + int64_t(2 * k) * m;
-      for (int64_t i = g; i < m; i += G) {
-        a2 = fma(ap[i], ap[i], a2);
-        b2 = fma(ap[m + i], ap[m + i], b2);
+    double a2 = 0.0, b2 = 0.0;
+    const double* const ap = Ac + int64_t(active ? 2 * k : 0) * m;
+    for (int w = 0; w < 256 && w < m; w += G) {  // G rows of every 256 at a time
+      double x2 = 0.0, y2 = 0.0, z = 0.0;
+      if (active) {
+        for (int64_t i = w + g; i < m; i += 256) {
+          x2 = fma(ap[i], ap[i], x2);
+          y2 = fma(ap[m + i], ap[m + i], y2);
+        }
       }
+      group_sum3<G>(x2, y2, z);
+      a2 += x2;
+      b2 += y2;
     }
-    group_sum3<G>(a2, b2, z);
     if (active && g < 2) sig[2 * k + g] = sqrt(g ? b2 : a2);
   }
   __syncthreads();
@@ -715,7 +811,7 @@ struct RingArgs {
   ulonglong2* ring;    // [2][N / 2][2][m + N] tagged doubles
   int* status;         // zero on entry; 1 not converged within max_sweeps, 2 a wait ran out
   int max_sweeps;
-  float tol;
+  double tol;
 };
 
 // One-sided Jacobi SVD, 32 <= N <= 256 and m <= 128 EA, N <= 128 EV: one block of 128 threads
@@ -735,7 +831,7 @@ struct RingArgs {
 // Every wait is bounded by g_barrier_limit_ns; a wait that runs out raises the abort flag
 // bar[2], which every other waiting block reads, and all blocks return with status 2.
 template <int EA, int EV>
-__global__ void __launch_bounds__(128) jacobi_ring_kernel(const RingArgs a) {
+__global__ void __launch_bounds__(128, 1) jacobi_ring_kernel(const RingArgs a) {
   __shared__ double part_s[3][128], tot_s[3], sig_s[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = a.m, n = a.n, N = a.N, L = N - 1, K = N / 2, k = blockIdx.x;
@@ -745,6 +841,16 @@ __global__ void __launch_bounds__(128) jacobi_ring_kernel(const RingArgs a) {
   // V's rows go round the warps in another order than A's, so that the warp with A's last
   // partial chunk is not the one with V's
   const int tv = (tid + 64) & 127;
+  // between two looks at a column that has not arrived: false when the wait is over in vain.
+  // The clock and the abort flag (a trip through L2) are read every 64 looks; with a limit
+  // of zero the first look is the last.
+  auto may_wait = [&](int spin, uint64_t& t0) {
+    if (limit != 0 && (spin & 63) != 63) return true;
+    const uint64_t now = global_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 >= limit) atomicExch(a.bar + 2, 1u);
+    return *abort_flag == 0u;
+  };
   double xs[EA], ys[EA], vx[EV], vy[EV];
   int p = k == 0 ? N - 1 : k, q = k == 0 ? 0 : L - k;
 #pragma unroll
@@ -861,18 +967,30 @@ __global__ void __launch_bounds__(128) jacobi_ring_kernel(const RingArgs a) {
             }
           }
           if (got) break;
-          if ((spin & 63) == 0) {
-            const uint64_t now = global_ns();
-            if (spin == 0) t0 = now;
-            if (now - t0 >= limit) atomicExch(a.bar + 2, 1u);
-            if (*abort_flag != 0u) { ok = false; break; }
-          }
+          if (!may_wait(spin, t0)) { ok = false; break; }
         }
       }
+      // V's columns were sent after A's: a first look now, checked where they are needed
+      bool have_v = true;
+      const ulonglong2* const vp_in = slot(tag & 1, k, 0) + m;
+      const ulonglong2* const vq_in = slot(tag & 1, k, 1) + m;
+      auto look_v = [&]() {
+        bool got = true;
+#pragma unroll
+        for (int e = 0; e < EV; ++e) {
+          const int i = tv + 128 * e;
+          if (i < N) {
+            if (k != 0 && k != last) got = get_tagged(vp_in + i, tag, vx[e]) && got;
+            got = get_tagged(vq_in + i, tag, vy[e]) && got;
+          }
+        }
+        return got;
+      };
+      if (moved) have_v = look_v();
       dots(al, be, ga);
       if (!totals(ok, al, be, ga)) { ok = false; break; }
       double c = 1.0, sn = 0.0;
-      const bool doit = jacobi_rotation(al, be, ga, floor2, a.tol, c, sn);
+      const bool doit = jacobi_rotation<false>(al, be, ga, floor2, a.tol, c, sn);
       any = any || doit;
       if (doit) {
 #pragma unroll
@@ -893,28 +1011,10 @@ __global__ void __launch_bounds__(128) jacobi_ring_kernel(const RingArgs a) {
           if (k != last) put_tagged(dq + i, ys[e], tag + 1);
         }
       }
-      if (moved) {
-        const ulonglong2* const bp = slot(tag & 1, k, 0) + m;
-        const ulonglong2* const bq = slot(tag & 1, k, 1) + m;
+      if (!have_v) {
         uint64_t t0 = 0;
-        for (int spin = 0;; ++spin) {
-          bool got = true;
-#pragma unroll
-          for (int e = 0; e < EV; ++e) {
-            const int i = tv + 128 * e;
-            if (i < N) {
-              if (k != 0 && k != last) got = get_tagged(bp + i, tag, vx[e]) && got;
-              got = get_tagged(bq + i, tag, vy[e]) && got;
-            }
-          }
-          if (got) break;
-          if ((spin & 63) == 0) {
-            const uint64_t now = global_ns();
-            if (spin == 0) t0 = now;
-            if (now - t0 >= limit) atomicExch(a.bar + 2, 1u);
-            if (*abort_flag != 0u) { ok = false; break; }
-          }
-        }
+        for (int spin = 0; !look_v(); ++spin)
+          if (!may_wait(spin, t0)) { ok = false; break; }
       }
       if (doit) {
 #pragma unroll
@@ -1144,10 +1244,10 @@ void launch_jacobi_small(const double* A, int64_t m, int n, int N, double* U, do
   const size_t sm = size_t(m * N + N * N) * sizeof(double);
   const int most = 200 * 1024 + 30 * 30 * int(sizeof(double));
   if (G == 16) {
-    jacobi_small_kernel<16><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, float(tol), status_dev);
+    jacobi_small_kernel<16><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, tol, status_dev);
   } else {
     ensure_smem_attr(reinterpret_cast<const void*>(jacobi_small_kernel<32>), most);
-    jacobi_small_kernel<32><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, float(tol), status_dev);
+    jacobi_small_kernel<32><<<1, threads, sm, s>>>(A, m, n, N, U, S, V, kJacobiSweeps, tol, status_dev);
   }
   TATRG_CUDA(cudaGetLastError());
 }
@@ -1183,7 +1283,7 @@ void launch_jacobi_ring(const double* A, int m, int n, int N, double* U, double*
   a.top = a.rot + kJacobiSweeps + 4;
   a.status = status_dev;
   a.max_sweeps = kJacobiSweeps;
-  a.tol = float(tol);
+  a.tol = tol;
   // registers for the columns: (A, V) chunks of 128 rows
   if (m <= 128) launch_ring<1, 1>(a, s);
   else if (m <= 256) launch_ring<2, 2>(a, s);
@@ -1226,8 +1326,10 @@ void cholesky_inverse(const double* G, int n, double* R, double* Rinv, int* stat
   check_extent(R, int64_t(n) * n - 1, sizeof(double), "cholesky output");
   check_extent(Rinv, int64_t(n) * n - 1, sizeof(double), "cholesky inverse");
   TATRG_CHECK(n >= 1 && n <= kCholMaxN, TATRG_EINVAL, "cholesky: n must be <= 168");
-  if (n <= 32) launch_chol<1>(G, n, R, Rinv, status_dev, first, shift_rel, s);
-  else if (n <= 64) launch_chol<4>(G, n, R, Rinv, status_dev, first, shift_rel, s);
+  if (n <= 32) {
+    chol_inverse_small_kernel<<<1, 128, 0, s>>>(G, n, R, Rinv, status_dev, first ? 1 : 0, shift_rel);
+    TATRG_CUDA(cudaGetLastError());
+  } else if (n <= 64) launch_chol<4>(G, n, R, Rinv, status_dev, first, shift_rel, s);
   else launch_chol<8>(G, n, R, Rinv, status_dev, first, shift_rel, s);
 }
 
