@@ -1,40 +1,9 @@
 #include "engine.cuh"
 
-#include <atomic>
 #include <cmath>
 #include <cstring>
 
 namespace tatrg {
-
-// The device's stream-ordered pool returns freed memory to the driver at every
-// synchronisation unless told to keep some, and mapping it again costs more than a small
-// building-block call computes (a 12 x 12 SVD, two reads of its spectrum: 330 us of which
-// the pool took most; a 0.5 GB operand of a contraction: 1 ms of 3.6).  So up to 8 GiB of
-// freed memory stay in the pool; what is above goes back at the next synchronisation, the
-// rest with the process or when a caller trims the device's default pool
-// (cudaMemPoolTrimTo).  A pool that already keeps more (tatrg_create raises it) is left.
-static void keep_pool_memory() {
-  constexpr uint64_t kKeep = uint64_t(8) << 30;
-  static std::atomic<uint64_t> done{0};  // a bit per device ordinal
-  int dev = 0;
-  TATRG_CUDA(cudaGetDevice(&dev));
-  const uint64_t bit = uint64_t(1) << (dev & 63);
-  if (dev < 64 && (done.load() & bit)) return;
-  cudaMemPool_t pool;
-  TATRG_CUDA(cudaDeviceGetDefaultMemPool(&pool, dev));
-  uint64_t keep = 0;
-  TATRG_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-  if (keep < kKeep) {
-    keep = kKeep;
-    TATRG_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-  }
-  done.fetch_or(bit);
-}
-
-Engine::Engine(cudaStream_t s) : s_(s) {
-  keep_pool_memory();
-  flag_.alloc(sizeof(int) * 4, s);
-}
 
 int keep_count(const std::vector<double>& v, double rel, int64_t cap) {
   if (v.empty() || !(v[0] > 0.0)) return 0;

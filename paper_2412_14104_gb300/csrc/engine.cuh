@@ -31,7 +31,7 @@ struct SvdResult {
 
 class Engine {
  public:
-  explicit Engine(cudaStream_t s);
+  explicit Engine(cudaStream_t s) : s_(s), flag_(sizeof(int) * 4, s) {}
   cudaStream_t stream() const { return s_; }
   Stats& stats() { return st_; }
 
