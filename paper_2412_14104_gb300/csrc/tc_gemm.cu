@@ -19,6 +19,8 @@
 #include <cuda_bf16.h>
 
 #include <atomic>
+#include <cmath>
+#include <cstring>
 #include <tuple>
 
 #include "kernels.cuh"
@@ -269,20 +271,70 @@ __device__ __forceinline__ constexpr uint32_t idesc() {
          (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 
-// float <-> double by IEEE-754 bit manipulation on the integer pipes: this GPU has few FP64
-// units, and a conversion on them costs as much as an FP64 add.  Values outside the
-// normal range of float (zero, subnormals, overflow, inf, nan) take the hardware
-// conversion.
-__device__ __forceinline__ double f2d_bits(float f) {
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t e = (u >> 23) & 0xFFu;
-  if (e == 0u || e == 255u) {
-    if ((u << 1) == 0u) return __longlong_as_double(int64_t(uint64_t(u) << 32));  // signed zero
-    return double(f);
-  }
-  return __longlong_as_double(int64_t((uint64_t(u & 0x80000000u) << 32) | (uint64_t(e + 896u) << 52) |
-                                      (uint64_t(u & 0x7FFFFFu) << 29)));
+// The double nearest to hi + lo, the bits of double(hi) + double(lo).  An SM of this GPU
+// completes two FP64 additions per clock, so the 16384 sums of an output tile held it for
+// 8192 clocks, a third of the tile's MMAs at K = 1024; this is about 20 FP32 and integer
+// instructions, 64 lanes or more of them per clock.  TwoSum gives s + e = hi + lo with
+// |e| <= ulp(s) / 2, so s, widened, is off by a whole number of double ulps, which is added
+// to its bits as an integer (below a power of two the ulp is half as large).
+__host__ __device__ __forceinline__ uint32_t f32_bits(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  uint32_t u;
+  memcpy(&u, &x, 4);
+  return u;
+#endif
 }
+__host__ __device__ __forceinline__ float bits_f32(uint32_t u) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(u);
+#else
+  float x;
+  memcpy(&x, &u, 4);
+  return x;
+#endif
+}
+__host__ __device__ __forceinline__ double sum_f32x2(float hi, float lo) {
+  const float s = hi + lo, bb = s - hi;
+  const float e = (hi - (s - bb)) + (lo - bb);
+  const uint32_t u = f32_bits(s), sign = u & 0x80000000u, ex = (u >> 23) & 0xFFu;
+  uint32_t top, low;
+  if (ex - 64u > 190u) {  // below 2^-63, inf, nan: the FP64 unit, but for exact zeros
+    if (hi != 0.0f || lo != 0.0f) return double(hi) + double(lo);
+    top = sign;
+    low = 0u;
+  } else {
+    const float d = bits_f32(f32_bits(e) ^ sign);  // > 0: away from zero
+    const float ulps = d * bits_f32((306u + ((d < 0.0f && (u & 0x7FFFFFu) == 0u) ? 1u : 0u) - ex) << 23);
+#ifdef __CUDA_ARCH__
+    const int n = __float2int_rn(ulps);
+#else
+    const int n = int(lrintf(ulps));
+#endif
+    const uint64_t w = ((uint64_t(((u & 0x7FFFFFFFu) >> 3) + 0x38000000u) << 32) | uint64_t(u << 29)) + uint64_t(int64_t(n));
+    top = uint32_t(w >> 32) | sign;
+    low = uint32_t(w);
+  }
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(int(top), int(low));
+#else
+  const uint64_t w = (uint64_t(top) << 32) | low;
+  double x;
+  memcpy(&x, &w, 8);
+  return x;
+#endif
+}
+// x 2^k: the exponent field moves while the result stays normal
+__device__ __forceinline__ double scale_exp2(double x, int k) {
+  const int top = __double2hiint(x);
+  const int ex = (top >> 20) & 0x7FF;
+  if (ex == 0 || ex == 0x7FF || ex + k <= 0 || ex + k >= 0x7FF) return ldexp(x, k);
+  return __hiloint2double(top + (k << 20), __double2loint(x));
+}
+// float nearest to a double by bit manipulation on the integer pipes: a conversion on the
+// few FP64 units costs as much as an FP64 add.  Values outside the normal range of float
+// (subnormals, overflow, inf, nan) take the hardware conversion.
 // round to nearest, ties to even
 __device__ __forceinline__ float d2f_bits(double x) {
   const uint64_t b = uint64_t(__double_as_longlong(x));
@@ -669,7 +721,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
 #pragma unroll
               for (int c = 0; c < 8; ++c) {
                 const int j = 8 * half + c;
-                double x = f2d_bits(__uint_as_float(vh[j])) + f2d_bits(__uint_as_float(vl[j]));
+                double x = sum_f32x2(__uint_as_float(vh[j]), __uint_as_float(vl[j]));
                 if (alpha != 1.0) x *= alpha;
                 stg[lane * 8 + (c ^ (lane & 7))] = x;
               }
@@ -704,7 +756,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
             for (int j = 0; j < 16; ++j) {
               if (16 * part + j < ncols) {
                 double* p = crow + co[j];
-                double x = f2d_bits(__uint_as_float(vh[j])) + f2d_bits(__uint_as_float(vl[j]));
+                double x = sum_f32x2(__uint_as_float(vh[j]), __uint_as_float(vl[j]));
                 if (alpha != 1.0) x *= alpha;
                 if (mode == 2) atomicAdd(p, x);
                 else if (mode == 1) *p = fma(beta, *p, x);
@@ -1319,8 +1371,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
           __syncwarp();
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
-            double x = f2d_bits(__uint_as_float(vh[c])) + f2d_bits(__uint_as_float(vl[c]));
-            x = ldexp(x, er + col_exp[cb + c]);
+            double x = scale_exp2(sum_f32x2(__uint_as_float(vh[c]), __uint_as_float(vl[c])), er + col_exp[cb + c]);
             if (alpha != 1.0) x *= alpha;
             stg[lane * 8 + (c ^ (lane & 7))] = x;
           }

@@ -135,3 +135,28 @@ def test_cholesky_breakdown_in_any_panel(torch, n, j):
     q = Q.cpu().numpy().ravel()[:200 * k].reshape(200, k)
     r = R.cpu().numpy().ravel()[:k * n].reshape(k, n)
     assert np.linalg.norm(q @ r - Y) <= 72 * n * EPS * np.linalg.norm(Y)
+
+
+@pytest.mark.parametrize("mode", [-1, 1, 2])
+@pytest.mark.parametrize("prec", [tg.TF32X3, tg.BF16X3, tg.BF16X6])
+def test_split_contraction_sums_two_floats_exactly(torch, prec, mode):
+    """The epilogue's hi + lo: row i has x_i in the first chain of K and y_i 128 elements on,
+    both exact in bf16, B is one there, so C is the double nearest to x_i + y_i, to the bit:
+    exponents far apart, cancellation, powers of two from below, exact zeros, tiny values."""
+    M, N, K = 1024, 144, 256
+    rng = np.random.default_rng(11)
+    man = rng.integers(128, 256, (2, M)) / 128.0 * rng.choice([-1.0, 1.0], (2, M))
+    e0 = rng.integers(-90, 60, M)
+    x = man[0] * 2.0 ** e0
+    y = man[1] * 2.0 ** (e0 - rng.integers(-3, 40, M))
+    x[::5] = np.sign(x[::5]) * 2.0 ** e0[::5]      # powers of two, y mostly below
+    y[::7], x[::11], y[::13] = 0.0, 0.0, -x[::13]  # zeros and cancellation
+    A, B = np.zeros((M, K)), np.zeros((K, N))
+    A[:, 0], A[:, 128], B[0], B[128] = x, y, 1.0, 1.0
+    C = torch.zeros((M, N), dtype=torch.float64, device="cuda")
+    tg.set_cta_pairs(mode)
+    try:
+        tg.contract([(M, K, N)], [(N, 1, 1)], [(K, 1, N)], _dev(torch, A), _dev(torch, B), C, precision=prec)
+    finally:
+        tg.set_cta_pairs(0)
+    assert np.array_equal(C.cpu().numpy(), np.repeat((x + y)[:, None], N, axis=1))
