@@ -86,17 +86,25 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
       : "memory");
   return ok != 0;
 }
-// bounded wait; false (and the error flag) when the deadline passes
+// bounded wait; false (and the error flag) after WAIT_NS.  The global timer is read once a
+// look has failed and every 16 looks from then on: it is slow to read, and the waits of the
+// load and MMA warps are on the path of every stage.
 template <bool CLUSTER = false>
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t deadline) {
-  while (!(CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity))) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  auto look = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+  if (look()) return true;
+  const uint64_t deadline = now_ns() + WAIT_NS;
+  while (true) {
+#pragma unroll 1
+    for (int i = 0; i < 16; ++i)
+      if (look()) return true;
     if (now_ns() > deadline) {
       atomicExch(&g_tc_error, 1);
       return false;
     }
   }
-  return true;
 }
+__device__ __forceinline__ bool all_lanes(bool p) { return __all_sync(0xffffffffu, p) != 0; }
 // CTA pairs (a cluster of two CTAs on two SMs sharing one MMA)
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -271,66 +279,29 @@ __device__ __forceinline__ constexpr uint32_t idesc() {
          (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 
-// The double nearest to hi + lo, the bits of double(hi) + double(lo).  An SM of this GPU
-// completes two FP64 additions per clock, so the 16384 sums of an output tile held it for
-// 8192 clocks, a third of the tile's MMAs at K = 1024; this is about 20 FP32 and integer
-// instructions, 64 lanes or more of them per clock.  TwoSum gives s + e = hi + lo with
-// |e| <= ulp(s) / 2, so s, widened, is off by a whole number of double ulps, which is added
-// to its bits as an integer (below a power of two the ulp is half as large).
-__host__ __device__ __forceinline__ uint32_t f32_bits(float x) {
-#ifdef __CUDA_ARCH__
-  return __float_as_uint(x);
-#else
-  uint32_t u;
-  memcpy(&u, &x, 4);
-  return u;
-#endif
+// The double nearest to s + e, of the floats that TwoSum made of hi + lo (|e| <= ulp(s) / 2):
+// the bits of double(hi) + double(lo).  An SM of this GPU completes two FP64 additions per
+// clock, so the 16384 sums of a 128 x 128 tile held it for 8192 clocks, a third of the tile's
+// MMAs at K = 1024; this is about 20 FP32 and integer instructions, 64 lanes or more of them
+// per clock.  s, widened, is off by a whole number of double ulps, which is added to its bits
+// as an integer (below a power of two the ulp is half as large).  `fp64` is raised for s
+// below 2^-63, inf and nan, whose sums the FP64 unit forms.
+__device__ __forceinline__ double widen_sum(uint32_t s, uint32_t e, bool& fp64) {
+  const uint32_t sign = s & 0x80000000u, mag = s & 0x7FFFFFFFu, ex = mag >> 23;
+  fp64 = fp64 || (ex - 64u > 190u && mag != 0u);
+  const float d = __uint_as_float(e ^ sign);  // > 0: away from zero
+  const uint32_t k = 306u + ((d < 0.0f && (s & 0x7FFFFFu) == 0u) ? 1u : 0u) - ex;
+  const int n = __float2int_rn(d * __uint_as_float(k << 23));  // 0 where s = 0, with e = 0
+  const uint64_t w = ((uint64_t(ex != 0u ? (mag >> 3) + 0x38000000u : 0u) << 32) | uint64_t(s << 29)) + uint64_t(int64_t(n));
+  return __hiloint2double(int(uint32_t(w >> 32) | sign), int(uint32_t(w)));
 }
-__host__ __device__ __forceinline__ float bits_f32(uint32_t u) {
-#ifdef __CUDA_ARCH__
-  return __uint_as_float(u);
-#else
-  float x;
-  memcpy(&x, &u, 4);
-  return x;
-#endif
-}
-__host__ __device__ __forceinline__ double sum_f32x2(float hi, float lo) {
-  const float s = hi + lo, bb = s - hi;
-  const float e = (hi - (s - bb)) + (lo - bb);
-  const uint32_t u = f32_bits(s), sign = u & 0x80000000u, ex = (u >> 23) & 0xFFu;
-  uint32_t top, low;
-  if (ex - 64u > 190u) {  // below 2^-63, inf, nan: the FP64 unit, but for exact zeros
-    if (hi != 0.0f || lo != 0.0f) return double(hi) + double(lo);
-    top = sign;
-    low = 0u;
-  } else {
-    const float d = bits_f32(f32_bits(e) ^ sign);  // > 0: away from zero
-    const float ulps = d * bits_f32((306u + ((d < 0.0f && (u & 0x7FFFFFu) == 0u) ? 1u : 0u) - ex) << 23);
-#ifdef __CUDA_ARCH__
-    const int n = __float2int_rn(ulps);
-#else
-    const int n = int(lrintf(ulps));
-#endif
-    const uint64_t w = ((uint64_t(((u & 0x7FFFFFFFu) >> 3) + 0x38000000u) << 32) | uint64_t(u << 29)) + uint64_t(int64_t(n));
-    top = uint32_t(w >> 32) | sign;
-    low = uint32_t(w);
-  }
-#ifdef __CUDA_ARCH__
-  return __hiloint2double(int(top), int(low));
-#else
-  const uint64_t w = (uint64_t(top) << 32) | low;
-  double x;
-  memcpy(&x, &w, 8);
-  return x;
-#endif
-}
-// x 2^k: the exponent field moves while the result stays normal
-__device__ __forceinline__ double scale_exp2(double x, int k) {
-  const int top = __double2hiint(x);
-  const int ex = (top >> 20) & 0x7FF;
-  if (ex == 0 || ex == 0x7FF || ex + k <= 0 || ex + k >= 0x7FF) return ldexp(x, k);
-  return __hiloint2double(top + (k << 20), __double2loint(x));
+// x 2^k by its exponent field, for x = 0, inf, nan or a normal x; `fp64` is raised where the
+// result is not normal
+__device__ __forceinline__ double scale_exp2(double x, int k, bool& fp64) {
+  const int top = __double2hiint(x), ex = (top >> 20) & 0x7FF;
+  const bool moves = ex != 0 && ex != 0x7FF;
+  fp64 = fp64 || (moves && uint32_t(ex + k - 1) >= 0x7FEu);
+  return __hiloint2double(moves ? top + (k << 20) : top, __double2loint(x));
 }
 // float nearest to a double by bit manipulation on the integer pipes: a conversion on the
 // few FP64 units costs as much as an FP64 add.  Values outside the normal range of float
@@ -358,6 +329,8 @@ struct TcArgs {
   double alpha, beta;
   int atomic;
   int n_contig;  // the C offset of output column n is n (the N modes run contiguously in C)
+  int vec;       // ... and every row of C starts on a 16-byte boundary
+  int scaled;    // alpha != 1
   double* C;
 };
 
@@ -387,6 +360,118 @@ __device__ __forceinline__ void two_sum_acc2(uint64_t& hi, uint64_t& lo, uint64_
   const uint64_t e = add2(sub2(hi, sub2(s, bb)), sub2(v, bb));
   lo = add2(lo, e);
   hi = s;
+}
+
+// The output of a warp goes through its 2 KB of shared memory in slices of 32 rows x 8
+// columns: a lane puts its row's eight doubles there as four 16-byte chunks (swizzled: eight
+// lanes cover all banks) and takes out chunk lane % 4 of rows lane / 4 + 8 i, so that four
+// lanes write 64 contiguous bytes of a row.
+__device__ __forceinline__ double2* stage_chunk(double* stg, int row, int chunk) {
+  return reinterpret_cast<double2*>(stg + row * 8) + (chunk ^ ((row >> 1) & 3));
+}
+// hi + lo of eight columns into the slice, with EXPS times 2^(exp_row + exps[column]).  What needs the FP64 unit is done in
+// a loop over shared memory, not in a branch per value: as predicated instructions that no
+// lane executes, the FP64 additions doubled the time of the whole output.
+template <bool EXPS>
+__device__ __forceinline__ void stage_sums(double* stg, int lane, const uint32_t (&hi)[8], const uint32_t (&lo)[8],
+                                           int scaled, double alpha, int exp_row, const int* exps) {
+  bool fp64 = false;
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    const uint64_t h = pk(hi[j], hi[j + 1]), l = pk(lo[j], lo[j + 1]);
+    const uint64_t s = add2(h, l), bb = sub2(s, h), e = add2(sub2(h, sub2(s, bb)), sub2(l, bb));
+    uint32_t s0, s1, e0, e1;
+    unpk(s, s0, s1);
+    unpk(e, e0, e1);
+    double x = widen_sum(s0, e0, fp64), y = widen_sum(s1, e1, fp64);
+    if (EXPS) {
+      x = scale_exp2(x, exp_row + exps[j], fp64);
+      y = scale_exp2(y, exp_row + exps[j + 1], fp64);
+    }
+    *stage_chunk(stg, lane, j >> 1) = make_double2(x, y);
+  }
+  if (__any_sync(0xffffffffu, fp64)) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      reinterpret_cast<uint2*>(stage_chunk(stg, lane, j >> 1))[j & 1] = make_uint2(hi[j], lo[j]);
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+      double* const at = reinterpret_cast<double*>(stage_chunk(stg, lane, j >> 1)) + (j & 1);
+      const float2 v = *reinterpret_cast<const float2*>(at);
+      const double x = double(v.x) + double(v.y);
+      *at = EXPS ? ldexp(x, exp_row + exps[j]) : x;
+    }
+  }
+  if (scaled) {
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      double2* const at = stage_chunk(stg, lane, j);
+      *at = make_double2(at->x * alpha, at->y * alpha);
+    }
+  }
+}
+// The C offset of row or column `flat`, below 2^31: no 64-bit division.
+__device__ __forceinline__ int64_t c_offset32(const DevModes& d, uint32_t flat) {
+  int64_t o = 0;
+#pragma unroll
+  for (int i = kMaxModes - 1; i >= 0; --i) {
+    if (i < d.n) {
+      const uint32_t e = uint32_t(d.ext[i]), q = flat / e;
+      o += int64_t(flat - q * e) * d.s1[i];
+      flat = q;
+    }
+  }
+  return o;
+}
+// Where a warp's rows and columns lie in C: its 32 rows (rows of them inside C), each lane
+// with the offsets of its own row and of the four it takes out of a slice.
+struct WarpRows {
+  int64_t own, out[4];
+  int rows;
+};
+__device__ __forceinline__ WarpRows warp_rows(const TcArgs& g, int64_t row0, int lane) {
+  WarpRows w;
+  w.rows = int(max(int64_t(0), min(int64_t(32), g.M - row0)));
+  w.own = lane < w.rows ? c_offset32(g.mC, uint32_t(row0 + lane)) : 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w.out[i] = __shfl_sync(0xffffffffu, w.own, (lane >> 2) + 8 * i);
+  return w;
+}
+__device__ __forceinline__ void put(double* p, double v, int mode, double beta) {
+  if (mode == 2) atomicAdd(p, v);
+  else *p = (mode == 1) ? fma(beta, *p, v) : v;
+}
+// Writes the staged slice: ncol of its eight columns, the first at output column n; co holds
+// the C offset of column n + c in lane c0 + c (unless the columns are contiguous in C).
+__device__ __forceinline__ void store_slice(const TcArgs& g, double* stg, int lane, const WarpRows& w, int64_t n,
+                                            int ncol, int64_t co, int c0, int mode) {
+  __syncwarp();
+  if (g.n_contig) {
+    const int c = lane & 3;
+    double* const col = g.C + n + 2 * c;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int row = (lane >> 2) + 8 * i;
+      const double2 v = *stage_chunk(stg, row, c);
+      if (row < w.rows) {
+        double* const p = col + w.out[i];
+        if (mode == 0 && g.vec && 2 * c + 1 < ncol) {
+          *reinterpret_cast<double2*>(p) = v;
+        } else {
+          if (2 * c < ncol) put(p, v.x, mode, g.beta);
+          if (2 * c + 1 < ncol) put(p + 1, v.y, mode, g.beta);
+        }
+      }
+    }
+  } else {  // a lane writes its row, a column an instruction (the rows may be contiguous in C)
+#pragma unroll 2
+    for (int j = 0; j < 8; ++j) {
+      const int64_t o = __shfl_sync(0xffffffffu, co, c0 + j);
+      const double2 v = *stage_chunk(stg, lane, j >> 1);
+      if (lane < w.rows && j < ncol) put(g.C + w.own + o, (j & 1) ? v.y : v.x, mode, g.beta);
+    }
+  }
+  __syncwarp();
 }
 
 // K stages ahead of the producer whose operand boxes are prefetched into L2 (0: none)
@@ -494,9 +579,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
   __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], peer_full[STAGES], acc_full[NBUF],
       acc_empty[NBUF], fin_bar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int64_t col_off[BN];
-  // per epilogue warp: a 32-row x 8-column slice of doubles (XOR-swizzled by row), through
-  // which the warp turns its row-per-lane values into row-contiguous stores
+  // per epilogue warp: a 32-row x 8-column slice of doubles on its way out (stage_chunk)
   __shared__ __align__(16) double epi_stage[EPI_WARPS * 32 * 8];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -545,7 +628,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
         for (int i = 0; i < w.nk; ++i, ++it) {
           if (TATRG_L2_PREFETCH > 0 && i + TATRG_L2_PREFETCH < w.nk) prefetch(i + TATRG_L2_PREFETCH);
           const int s = it % STAGES, round = it / STAGES;
-          if (round > 0 && !mbar_wait<CLU>(&empty_bar[s], (round - 1) & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+          if (round > 0 && !mbar_wait<CLU>(&empty_bar[s], (round - 1) & 1)) { ok = false; break; }
           uint8_t* st = smem + s * STAGE;
           mbar_expect_tx(&full_bar[s], STAGE);  // FORM 2: half of B comes from the other CTA
           const int kx = (w.kb0 + i) * KELEM;
@@ -561,9 +644,8 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
         }
       }
       // drain: the last loads issued into each stage must have landed before the CTA exits
-      const uint64_t drain = now_ns() + WAIT_NS;
       for (int i = max(0, it - STAGES); i < it; ++i)
-        mbar_wait(&full_bar[i % STAGES], (i / STAGES) & 1, drain);
+        mbar_wait(&full_bar[i % STAGES], (i / STAGES) & 1);
     }
   } else if (warp == 1 && (!PAIR || rank == 0)) {
     if (lane == 0) {
@@ -575,14 +657,14 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
         const int nchunks = (w.nk + KC - 1) / KC;
         for (int c = 0; c < nchunks && ok; ++c, ++cc) {
           const int b = cc % NBUF, use = cc / NBUF;
-          if (use > 0 && !mbar_wait<PAIR>(&acc_empty[b], (use - 1) & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+          if (use > 0 && !mbar_wait<PAIR>(&acc_empty[b], (use - 1) & 1)) { ok = false; break; }
           tc_fence_after();
           const uint32_t acc = tmem + uint32_t(b * BN);
           const int i_end = min(w.nk, (c + 1) * KC);
           for (int i = c * KC; i < i_end; ++i, ++it) {
             const int s = it % STAGES, round = it / STAGES;
-            if (!mbar_wait(&full_bar[s], round & 1, now_ns() + WAIT_NS)) { ok = false; break; }
-            if (PAIR && !mbar_wait<true>(&peer_full[s], round & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+            if (!mbar_wait(&full_bar[s], round & 1)) { ok = false; break; }
+            if (PAIR && !mbar_wait<true>(&peer_full[s], round & 1)) { ok = false; break; }
             tc_fence_after();
             // descriptors of the stage's slices, formed once (the issuing thread is on the
             // critical path of every MMA)
@@ -609,7 +691,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
       }
       // drain: every MMA issued by this thread completes before TMEM is released
       mma_commit<CG>(&fin_bar);
-      mbar_wait<PAIR>(&fin_bar, 0, now_ns() + WAIT_NS);
+      mbar_wait<PAIR>(&fin_bar, 0);
     }
   } else if (warp == 1) {  // PAIR, rank 1
     if (lane == 0) {
@@ -621,13 +703,13 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
         const Unit w = unit_of<TILE_M>(g, u);
         for (int i = 0; i < w.nk; ++i, ++it) {
           const int s = it % STAGES, round = it / STAGES;
-          if (!mbar_wait(&full_bar[s], round & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+          if (!mbar_wait(&full_bar[s], round & 1)) { ok = false; break; }
           mbar_arrive_remote(peer0 + uint32_t(s * sizeof(uint64_t)));
         }
       }
       // the first CTA's final commit also arrives here: its MMAs into this CTA's tensor
       // memory are complete before the memory is released
-      mbar_wait<true>(&fin_bar, 0, now_ns() + WAIT_NS);
+      mbar_wait<true>(&fin_bar, 0);
     }
   } else {
     // epilogue warps 2..17: TMEM lane quarter q = warp % 4 (the lanes a warp may access),
@@ -635,7 +717,6 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
     // [NBUF*BN, NBUF*BN + BN) (hi) and [NBUF*BN + BN, NBUF*BN + 2*BN) (lo), so the drain
     // needs few registers.
     const int q = warp & 3, h = (warp - 2) >> 2;
-    const int row = int(rank) * TC_BM + q * 32 + lane;  // row of the tile
     const uint32_t lanes = tmem + (uint32_t(q * 32) << 16);
     const uint32_t t_hi = lanes + uint32_t(NBUF * BN + h * 32);
     const uint32_t t_lo = lanes + uint32_t(NBUF * BN + BN + h * 32);
@@ -645,19 +726,11 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
 #pragma unroll 1
     for (int u = first; u < units && ok; u += stride) {
       const Unit w = unit_of<TILE_M>(g, u);
-      // per-column C offsets of this tile (the previous tile's stores are done with them)
-      asm volatile("bar.sync 1, %0;" ::"r"(EPI_WARPS * 32) : "memory");
-      for (int j = threadIdx.x - 64; j < BN; j += EPI_WARPS * 32) {
-        int64_t a = 0, c = 0;
-        if (w.n0 + j < g.N) mode_offsets(g.nC, w.n0 + j, a, c);
-        col_off[j] = c;
-      }
-      asm volatile("bar.sync 1, %0;" ::"r"(EPI_WARPS * 32) : "memory");
       const int nchunks = (w.nk + KC - 1) / KC;
 #pragma unroll 1
       for (int c = 0; c < nchunks; ++c, ++cc) {
         const int b = cc % NBUF, use = cc / NBUF;
-        ok = __all_sync(0xffffffffu, (ok && mbar_wait<PAIR>(&acc_full[b], use & 1, now_ns() + WAIT_NS)) ? 1 : 0) != 0;
+        ok = all_lanes(ok && (lane != 0 || mbar_wait<PAIR>(&acc_full[b], use & 1)));
         if (!ok) break;
         tc_fence_after();
         const uint32_t ta = lanes + uint32_t(b * BN + h * 32);
@@ -698,72 +771,21 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
       // one decision for all epilogue warps (a wait that ran out in any of them stops all)
       ok = epilogue_all(ok);
       if (ok) {
-        const bool in_rows = (w.m0 + row) < g.M;
-        int64_t roff = 0, dummy = 0;
-        if (in_rows) mode_offsets(g.mC, w.m0 + row, dummy, roff);
-        const double alpha = g.alpha, beta = g.beta;
-        const int mode = g.atomic ? 2 : (beta != 0.0 ? 1 : 0);
-        if (g.n_contig && mode != 2) {
-          // coalesced: each slice of 8 columns goes through shared memory so that eight
-          // lanes write 64 contiguous bytes of one row (four rows per store instruction)
-          double* const stg = epi_stage + (warp - 2) * 256;
+        const WarpRows wr = warp_rows(g, w.m0 + int(rank) * TC_BM + q * 32, lane);
+        const int mode = g.atomic ? 2 : (g.beta != 0.0 ? 1 : 0);
+        double* const stg = epi_stage + (warp - 2) * 256;
+        const int64_t nw = w.n0 + h * 32;  // the warp's first output column
+        const int64_t co = nw + lane < g.N && !g.n_contig ? c_offset32(g.nC, uint32_t(nw + lane)) : 0;
 #pragma unroll
-          for (int part = 0; part < 2; ++part) {
-            if (w.n0 + h * 32 + 16 * part >= g.N) break;  // the rest of this warp's columns are padding
-            uint32_t vh[16], vl[16];
-            tmem_ld16_nowait(t_hi + uint32_t(16 * part), vh);
-            tmem_ld16_nowait(t_lo + uint32_t(16 * part), vl);
-            tmem_wait_ld();
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              if (w.n0 + h * 32 + 16 * part + 8 * half >= g.N) break;
-              __syncwarp();
-#pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                const int j = 8 * half + c;
-                double x = sum_f32x2(__uint_as_float(vh[j]), __uint_as_float(vl[j]));
-                if (alpha != 1.0) x *= alpha;
-                stg[lane * 8 + (c ^ (lane & 7))] = x;
-              }
-              __syncwarp();
-              const int cb = h * 32 + 16 * part + 8 * half;  // tile column of the slice
-              const int c = lane & 7;
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int r = (lane >> 3) + 4 * i;  // row of the warp's 32
-                const int64_t rb = __shfl_sync(0xffffffffu, roff, r);
-                const int rin = __shfl_sync(0xffffffffu, in_rows ? 1 : 0, r);
-                const double v = stg[r * 8 + (c ^ (r & 7))];
-                if (rin && w.n0 + cb + c < g.N) {
-                  double* p = g.C + rb + col_off[cb + c];
-                  *p = (mode == 1) ? fma(beta, *p, v) : v;
-                }
-              }
-            }
-          }
-        } else {
-          double* const crow = g.C + roff;
-          const int64_t rem_ = g.N - (w.n0 + h * 32);
-          const int ncols = !in_rows ? 0 : (rem_ < 32 ? int(rem_) : 32);
-#pragma unroll
-          for (int part = 0; part < 2; ++part) {
-            uint32_t vh[16], vl[16];
-            tmem_ld16_nowait(t_hi + uint32_t(16 * part), vh);
-            tmem_ld16_nowait(t_lo + uint32_t(16 * part), vl);
-            tmem_wait_ld();
-            const int64_t* const co = col_off + h * 32 + 16 * part;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              if (16 * part + j < ncols) {
-                double* p = crow + co[j];
-                double x = sum_f32x2(__uint_as_float(vh[j]), __uint_as_float(vl[j]));
-                if (alpha != 1.0) x *= alpha;
-                if (mode == 2) atomicAdd(p, x);
-                else if (mode == 1) *p = fma(beta, *p, x);
-                else *p = x;
-              }
-            }
-          }
+        for (int part = 0; part < 4; ++part) {
+          const int ncol = int(min(int64_t(8), g.N - nw - 8 * part));
+          if (ncol <= 0) break;  // the rest of this warp's columns are padding
+          uint32_t vh[8], vl[8];
+          tmem_ld8_nowait(t_hi + uint32_t(8 * part), vh);
+          tmem_ld8_nowait(t_lo + uint32_t(8 * part), vl);
+          tmem_wait_ld();
+          stage_sums<false>(stg, lane, vh, vl, g.scaled, g.alpha, 0, nullptr);
+          store_slice(g, stg, lane, wr, nw + 8 * part, ncol, co, 8 * part, mode);
         }
       }
     }
@@ -1195,7 +1217,6 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full_bar[OZ_STAGES], empty_bar[OZ_STAGES], acc_full[2], acc_empty[2], fin_bar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int64_t col_off[OZ_BN];
   __shared__ int col_exp[OZ_BN];
   __shared__ __align__(16) double epi_stage[EPI_WARPS * 32 * 8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1227,7 +1248,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
         const Unit w = oz_unit_of(g, u);
         for (int i = 0; i < w.nk; ++i, ++it) {
           const int s = it % OZ_STAGES, round = it / OZ_STAGES;
-          if (round > 0 && !mbar_wait(&empty_bar[s], (round - 1) & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+          if (round > 0 && !mbar_wait(&empty_bar[s], (round - 1) & 1)) { ok = false; break; }
           uint8_t* st = smem + s * OZ_STAGE;
           mbar_expect_tx(&full_bar[s], OZ_STAGE);
           const int kx = (w.kb0 + i) * OZ_KELEM;
@@ -1238,8 +1259,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
           }
         }
       }
-      const uint64_t drain = now_ns() + WAIT_NS;
-      for (int i = max(0, it - OZ_STAGES); i < it; ++i) mbar_wait(&full_bar[i % OZ_STAGES], (i / OZ_STAGES) & 1, drain);
+      for (int i = max(0, it - OZ_STAGES); i < it; ++i) mbar_wait(&full_bar[i % OZ_STAGES], (i / OZ_STAGES) & 1);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -1251,13 +1271,13 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
         const int nchunks = (w.nk + OZ_KC - 1) / OZ_KC;
         for (int c = 0; c < nchunks && ok; ++c, ++cc) {
           const int b = cc & 1, use = cc >> 1;
-          if (use > 0 && !mbar_wait(&acc_empty[b], (use - 1) & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+          if (use > 0 && !mbar_wait(&acc_empty[b], (use - 1) & 1)) { ok = false; break; }
           tc_fence_after();
           const uint32_t acc = tmem + uint32_t(b * ACC_COLS);
           const int i_end = min(w.nk, (c + 1) * OZ_KC);
           for (int i = c * OZ_KC; i < i_end; ++i, ++it) {
             const int s = it % OZ_STAGES, round = it / OZ_STAGES;
-            if (!mbar_wait(&full_bar[s], round & 1, now_ns() + WAIT_NS)) { ok = false; break; }
+            if (!mbar_wait(&full_bar[s], round & 1)) { ok = false; break; }
             tc_fence_after();
             const uint64_t d0 = sdesc_sw64(smem_u32(smem + s * OZ_STAGE));
             uint64_t ad[OZ_NS], bd[OZ_NS];
@@ -1280,12 +1300,11 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
         }
       }
       mma_commit<1>(&fin_bar);
-      mbar_wait(&fin_bar, 0, now_ns() + WAIT_NS);
+      mbar_wait(&fin_bar, 0);
     }
   } else {
     // epilogue warps 2..17: lane quarter q, column quarter h (16 of the 64 columns)
     const int q = warp & 3, h = (warp - 2) >> 2;
-    const int row = q * 32 + lane;
     const uint32_t lanes = tmem + (uint32_t(q * 32) << 16);
     int cc = 0;
     bool ok = true;
@@ -1294,9 +1313,6 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
       const Unit w = oz_unit_of(g, u);
       asm volatile("bar.sync 1, %0;" ::"r"(EPI_WARPS * 32) : "memory");
       for (int j = threadIdx.x - 64; j < OZ_BN; j += EPI_WARPS * 32) {
-        int64_t a = 0, c = 0;
-        if (w.n0 + j < g.N) mode_offsets(g.nC, w.n0 + j, a, c);
-        col_off[j] = c;
         const int e = args.eb[w.n0 + j];
         col_exp[j] = e == OZ_EXP_NONE ? 0 : e;
       }
@@ -1305,7 +1321,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
 #pragma unroll 1
       for (int c = 0; c < nchunks; ++c, ++cc) {
         const int b = cc & 1, use = cc >> 1;
-        ok = __all_sync(0xffffffffu, (ok && mbar_wait(&acc_full[b], use & 1, now_ns() + WAIT_NS)) ? 1 : 0) != 0;
+        ok = all_lanes(ok && (lane != 0 || mbar_wait(&acc_full[b], use & 1)));
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
@@ -1352,43 +1368,23 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
       }
       ok = epilogue_all(ok);
       if (ok) {
-        const bool in_rows = (w.m0 + row) < g.M;
-        int64_t roff = 0, dummy = 0;
-        if (in_rows) mode_offsets(g.mC, w.m0 + row, dummy, roff);
-        const int er0 = args.ea[w.m0 + row];
+        const WarpRows wr = warp_rows(g, w.m0 + q * 32, lane);
+        const int er0 = args.ea[w.m0 + q * 32 + lane];
         const int er = (er0 == OZ_EXP_NONE ? 0 : er0) - 14;
-        const double alpha = g.alpha, beta = g.beta;
-        const int mode = g.atomic ? 2 : (beta != 0.0 ? 1 : 0);
+        const int mode = g.atomic ? 2 : (g.beta != 0.0 ? 1 : 0);
         double* const stg = epi_stage + (warp - 2) * 256;
+        const int64_t nw = w.n0 + h * 16;
+        const int64_t co = lane < 16 && nw + lane < g.N && !g.n_contig ? c_offset32(g.nC, uint32_t(nw + lane)) : 0;
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
-          const int cb = h * 16 + part * 8;  // tile column of the slice
-          if (w.n0 + cb >= g.N) break;
+          const int ncol = int(min(int64_t(8), g.N - nw - 8 * part));
+          if (ncol <= 0) break;
           uint32_t vh[8], vl[8];
-          tmem_ld8_nowait(lanes + uint32_t(HI + cb), vh);
-          tmem_ld8_nowait(lanes + uint32_t(LO + cb), vl);
+          tmem_ld8_nowait(lanes + uint32_t(HI + h * 16 + 8 * part), vh);
+          tmem_ld8_nowait(lanes + uint32_t(LO + h * 16 + 8 * part), vl);
           tmem_wait_ld();
-          __syncwarp();
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            double x = scale_exp2(sum_f32x2(__uint_as_float(vh[c]), __uint_as_float(vl[c])), er + col_exp[cb + c]);
-            if (alpha != 1.0) x *= alpha;
-            stg[lane * 8 + (c ^ (lane & 7))] = x;
-          }
-          __syncwarp();
-          const int c = lane & 7;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = (lane >> 3) + 4 * i;
-            const int64_t rb = __shfl_sync(0xffffffffu, roff, r);
-            const int rin = __shfl_sync(0xffffffffu, in_rows ? 1 : 0, r);
-            const double v = stg[r * 8 + (c ^ (r & 7))];
-            if (rin && w.n0 + cb + c < g.N) {
-              double* p = g.C + rb + col_off[cb + c];
-              if (mode == 2) atomicAdd(p, v);
-              else *p = (mode == 1) ? fma(beta, *p, v) : v;
-            }
-          }
+          stage_sums<true>(stg, lane, vh, vl, g.scaled, g.alpha, er, col_exp + h * 16 + 8 * part);
+          store_slice(g, stg, lane, wr, nw + 8 * part, ncol, co, 8 * part, mode);
         }
       }
     }
@@ -1597,6 +1593,19 @@ TcChoice tuned_choice(int prec, int64_t M, int64_t N, int64_t K, int n_contig, b
 }
 }  // namespace
 
+// How the kernels write C: the offset of column n equals n when the N modes chain
+// contiguously in C; 16-byte stores of column pairs then need every row on that boundary.
+static void output_layout(const GemmDesc& d, double* C, TcArgs& a) {
+  bool contig = d.n.n >= 1 && d.n.s1[d.n.n - 1] == 1;
+  for (int i = 0; contig && i + 1 < d.n.n; ++i) contig = d.n.s1[i] == d.n.s1[i + 1] * d.n.ext[i + 1];
+  bool vec = contig && reinterpret_cast<uintptr_t>(C) % 16 == 0;
+  for (int i = 0; vec && i < d.m.n; ++i) vec = d.m.s1[i] % 2 == 0;
+  a.C = C;
+  a.n_contig = contig ? 1 : 0;
+  a.vec = vec ? 1 : 0;
+  a.scaled = d.alpha != 1.0 ? 1 : 0;
+}
+
 void gemm_tc(const GemmDesc& d, const double* A, const double* B, double* C, int prec,
              cudaStream_t s, Stats* st, const GaussSrc* gen_b) {
   TATRG_CHECK(prec >= 1 && prec <= 3, TATRG_EINVAL, "gemm_tc: precision must be TF32X3, BF16X3 or BF16X6");
@@ -1677,13 +1686,7 @@ void gemm_tc(const GemmDesc& d, const double* A, const double* B, double* C, int
   a.nkb = nkb;
   a.alpha = d.alpha;
   a.beta = d.beta;
-  {
-    // C offset of column n equals n when the N modes chain contiguously in C
-    bool contig = d.n.n >= 1 && d.n.s1[d.n.n - 1] == 1;
-    for (int i = 0; contig && i + 1 < d.n.n; ++i) contig = d.n.s1[i] == d.n.s1[i + 1] * d.n.ext[i + 1];
-    a.n_contig = contig ? 1 : 0;
-  }
-  a.C = C;
+  output_layout(d, C, a);
   a.ntiles = int(Np / BN);
   // one launch of configuration (tile form, split): C is rewritten whole (zeroed first when
   // K is split, the CTAs then add their partial sums)
@@ -1794,8 +1797,7 @@ void gemm_oz(const GemmDesc& d, const double* A, const double* B, double* C, cud
   g.nkb = int(Kp / OZ_KELEM);
   g.alpha = d.alpha;
   g.beta = d.beta;
-  g.n_contig = 0;
-  g.C = C;
+  output_layout(d, C, g);
   g.mtiles = int(Mp / TC_BM);
   g.ntiles = int(Np / OZ_BN);
   const int64_t tiles = int64_t(g.mtiles) * g.ntiles;
