@@ -83,6 +83,7 @@ def lib():
             "tatrg_philox_words": [U64, U32, U32, U64, I64, P, P],
             "tatrg_set_barrier_limit_ns": [ctypes.c_longlong],
             "tatrg_set_cta_pairs": [I],
+            "tatrg_release_memory": [],
         }
         for name, args in sig.items():
             f = getattr(L, name)
@@ -362,6 +363,12 @@ def set_cta_pairs(mode):
     """Tile form of the split-precision contractions: 0 autotuned, 1 CTA pairs, 2 multicast
     clusters wherever they apply (M >= 1024), -1 single CTAs only."""
     _check(lib().tatrg_set_cta_pairs(int(mode)))
+
+
+def release_memory():
+    """Gives the working memory that the building-block calls keep (at most 2 GiB on each
+    device) back to the driver."""
+    _check(lib().tatrg_release_memory())
 
 
 def lnz_function(chi, r, q=2, method=TRIAD, precision=FP64, seed=0, d=4, nsteps=8):

@@ -1753,6 +1753,11 @@ void tatrg_destroy(tatrg_ctx* ctx) {
   if (!ctx) return;
   cudaStreamSynchronize(ctx->stream);
   delete ctx;
+  trim_block_memory();
+}
+
+tatrg_status tatrg_release_memory(void) {
+  return guard(nullptr, [&] { trim_block_memory(); });
 }
 
 tatrg_status tatrg_gaussian(unsigned long long seed, uint32_t sid, uint32_t replica, int64_t rows,
@@ -1794,6 +1799,7 @@ tatrg_status tatrg_contract_sketch(const tatrg_contraction* c, int precision, co
     TATRG_CHECK(precision >= 1 && precision <= 3, TATRG_EINVAL,
                 "tatrg_contract_sketch: needs a split precision (1, 2 or 3)");
     const GemmDesc g = desc_of(c);
+    BlockMemory memory;
     Engine e(static_cast<cudaStream_t>(stream));
     e.prec = precision;
     const GaussSrc gs{seed, sid, replica};
@@ -1810,6 +1816,7 @@ tatrg_status tatrg_contract(const tatrg_contraction* c, int precision, const dou
     TATRG_CHECK(c && A && B && C, TATRG_EINVAL, "tatrg_contract: null argument");
     TATRG_CHECK(precision >= 0 && precision <= 4, TATRG_EINVAL, "tatrg_contract: bad precision");
     const GemmDesc g = desc_of(c);
+    BlockMemory memory;
     Engine e(static_cast<cudaStream_t>(stream));
     e.prec = precision;
     e.gemm(g, A, B, C);
@@ -1826,6 +1833,7 @@ tatrg_status tatrg_orth(int precision, int64_t m, int64_t n, const double* Y, do
     TATRG_CHECK(Y && Q && R && k && m >= n && n >= 1 && n <= 1024, TATRG_EINVAL, "tatrg_orth: bad argument");
     TATRG_CHECK(precision >= 0 && precision <= 4, TATRG_EINVAL, "tatrg_orth: bad precision");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    BlockMemory memory;
     Engine e(s);
     e.prec = precision;
     OrthResult o = e.orth(Y, m, n);
@@ -1840,6 +1848,7 @@ tatrg_status tatrg_svd(int64_t m, int64_t n, const double* A, double* U, double*
   return guard(nullptr, [&] {
     TATRG_CHECK(A && U && S && V && m >= n && n >= 1 && n <= 1024, TATRG_EINVAL, "tatrg_svd: bad argument");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    BlockMemory memory;
     Engine e(s);
     SvdResult r = e.svd(A, m, n);
     // a failed factorisation leaves the caller's arrays as they were

@@ -160,3 +160,46 @@ def test_split_contraction_sums_two_floats_exactly(torch, prec, mode):
     finally:
         tg.set_cta_pairs(0)
     assert np.array_equal(C.cpu().numpy(), np.repeat((x + y)[:, None], N, axis=1))
+
+
+def test_block_memory_is_bounded_and_given_back(torch):
+    """The building blocks' pool: at most 2 GiB (and the driver's granularity) kept after a call
+    that used 2.4 GB, nothing after release_memory(), and calls of two threads on two streams."""
+    import threading
+    M, N, K = 65536, 256, 4608  # 2.4 GB of packed operands in 3xTF32
+    A, B = torch.randn((M, K), dtype=torch.float64, device="cuda"), torch.randn((K, N), dtype=torch.float64, device="cuda")
+    C = torch.empty((M, N), dtype=torch.float64, device="cuda")
+    modes = [(M, K, N)], [(N, 1, 1)], [(K, 1, N)]
+    small = [(2304, K, N)], [(N, 1, 1)], [(K, 1, N)]
+    tg.contract(*small, A, B, C, precision=tg.TF32X3)
+    tg.release_memory()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    tg.contract(*modes, A, B, C, precision=tg.TF32X3)
+    torch.cuda.synchronize()
+    assert free0 - torch.cuda.mem_get_info()[0] <= (2 << 30) + (64 << 20)
+    tg.release_memory()
+    assert free0 - torch.cuda.mem_get_info()[0] <= 64 << 20
+    want = (A[:2304] @ B).cpu().numpy()
+    err = []
+
+    def work():
+        try:
+            s = torch.cuda.Stream()
+            out = torch.empty((2304, N), dtype=torch.float64, device="cuda")
+            s.wait_stream(torch.cuda.default_stream())
+            for _ in range(8):
+                tg.contract(*small, A, B, out, precision=tg.BF16X6, stream=s)
+                got = out.cpu().numpy()
+                err.append(np.max(np.abs(got - want)) / np.max(np.abs(want)))
+                tg.release_memory()
+        except Exception as e:  # the assertion below reports it
+            err.append(e)
+
+    threads = [threading.Thread(target=work) for _ in range(2)]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(err) == 16 and all(isinstance(e, float) and e < 1e-6 for e in err), err
