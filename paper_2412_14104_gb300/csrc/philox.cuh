@@ -42,6 +42,19 @@ __device__ __forceinline__ double u53(uint32_t a, uint32_t b) {
   return (double(a >> 5) * 67108864.0 + double(b >> 6) + 0.5) * (1.0 / 9007199254740992.0);
 }
 
+// float(u53(a, b)), to the bit, on the integer pipes (an SM completes two FP64 instructions
+// per clock, and the conversions and sums of u53 are eight): u53 = V 2^-54 with the odd
+// 54-bit V = 2 N + 1, which double rounds to 53 bits (a tie, to even) where it has 54.
+__device__ __forceinline__ float u53_f32(uint32_t a, uint32_t b) {
+  const uint64_t n = (uint64_t(a >> 5) << 26) | (b >> 6);
+  uint64_t v = (n >> 52) ? (n + (n & 1)) << 1 : 2 * n + 1;
+  const int lz = __clzll((long long)v);  // 9..63, or 9 after a carry to 2^54
+  v <<= lz;
+  // 32 leading bits, the last one standing for all below it: rounds to 24 as V does
+  const float f = __uint2float_rn(uint32_t(v >> 32) | (uint32_t(v) != 0u ? 1u : 0u));
+  return f * __uint_as_float(uint32_t(127 - 22 - lz) << 23);
+}
+
 // The pair (z0, z1) of counter block p with Box-Muller evaluated in float arithmetic
 // (relative error ~1e-7): for sketches that feed split-precision contractions, whose
 // operands are rounded to two tensor-core numbers (~2^-22 relative) anyway.  The uniforms
@@ -50,7 +63,7 @@ __device__ __forceinline__ void gauss_pair_f32(uint64_t seed, uint32_t sid, uint
                                                int64_t p, float& z0, float& z1) {
   uint32_t w[4];
   philox4x32_10(seed, sid, replica, p, w);
-  const float u1 = float(u53(w[0], w[1])), u2 = float(u53(w[2], w[3]));
+  const float u1 = u53_f32(w[0], w[1]), u2 = u53_f32(w[2], w[3]);
   const float rad = sqrtf(-2.0f * logf(u1));
   float sn, cs;
   sincospif(2.0f * u2, &sn, &cs);  // angle 2 pi u2, reduced exactly in units of pi

@@ -303,20 +303,30 @@ __device__ __forceinline__ double scale_exp2(double x, int k, bool& fp64) {
   fp64 = fp64 || (moves && uint32_t(ex + k - 1) >= 0x7FEu);
   return __hiloint2double(moves ? top + (k << 20) : top, __double2loint(x));
 }
-// float nearest to a double by bit manipulation on the integer pipes: a conversion on the
-// few FP64 units costs as much as an FP64 add.  Values outside the normal range of float
-// (subnormals, overflow, inf, nan) take the hardware conversion.
-// round to nearest, ties to even
+// The float nearest to a double (ties to even) on the integer pipes alone: a conversion
+// occupies the few FP64 units as long as an FP64 add does, also as a predicated instruction
+// that no lane executes.
 __device__ __forceinline__ float d2f_bits(double x) {
   const uint64_t b = uint64_t(__double_as_longlong(x));
-  if ((b << 1) == 0u) return __uint_as_float(uint32_t(b >> 32));  // signed zero
-  const int e = int((b >> 52) & 0x7FFu) - 896;                     // biased float exponent
-  if (e <= 0 || e >= 255) return __double2float_rn(x);
-  const uint64_t m = b & 0xFFFFFFFFFFFFFull;
-  uint32_t f = (uint32_t(b >> 32) & 0x80000000u) | (uint32_t(e) << 23) | uint32_t(m >> 29);
-  const uint64_t rem = m & 0x1FFFFFFFull, half = 0x10000000ull;
-  if (rem > half || (rem == half && (f & 1u))) f += 1u;  // a carry into the exponent rounds correctly
-  return __uint_as_float(f);
+  const uint32_t sign = uint32_t(b >> 32) & 0x80000000u;
+  const int e = int((b >> 52) & 0x7FFu) - 896;  // biased float exponent
+  if (uint32_t(e - 1) >= 254u) {                // not a normal float
+    const uint64_t m = b & 0xFFFFFFFFFFFFFull;
+    if (e >= 255) return __uint_as_float(e == 1151 && m != 0 ? 0x7FFFFFFFu : sign | 0x7F800000u);
+    if (e < -24) return __uint_as_float(sign);  // below half of the smallest subnormal (or zero)
+    const int sh = 30 - e;                      // 30..54
+    const uint64_t full = m | (uint64_t(1) << 52), half = uint64_t(1) << (sh - 1);
+    uint32_t f = uint32_t(full >> sh);
+    const uint64_t rem = full & ((uint64_t(1) << sh) - 1);
+    if (rem > half || (rem == half && (f & 1u))) f += 1u;
+    return __uint_as_float(sign | f);
+  }
+  // 29 bits are dropped; a carry into the exponent rounds correctly
+  const uint32_t lo = uint32_t(b), hi = uint32_t(b >> 32);
+  uint32_t f = (uint32_t(e) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  const uint32_t rem = lo & 0x1FFFFFFFu;
+  f += (rem + (f & 1u) > 0x10000000u) ? 1u : 0u;
+  return __uint_as_float(sign | f);
 }
 
 struct TcArgs {
@@ -809,11 +819,27 @@ __device__ __forceinline__ float tf32_rna(float x) {
   return __uint_as_float(r);
 }
 
+// The source offset of row or K element `flat`, below 2^31: no 64-bit division.
+__device__ __forceinline__ int64_t src_offset32(const DevModes& d, uint32_t flat) {
+  int64_t o = 0;
+#pragma unroll
+  for (int i = kMaxModes - 1; i >= 0; --i) {
+    if (i < d.n) {
+      const uint32_t e = uint32_t(d.ext[i]), q = flat / e;
+      o += int64_t(flat - q * e) * d.s0[i];
+      flat = q;
+    }
+  }
+  return o;
+}
+
 // One block packs a strip of PK_R rows x PK_K K-elements per iteration (grid-stride over
 // strips).  The row and K offsets of the strip are decomposed once into shared memory.
-// K-contiguous sources are read and written with the lanes along K (no staging);
-// row-contiguous sources are read with the lanes along the rows into a shared tile and
-// written from it with the lanes along K.
+// K-contiguous sources are read with the lanes along K; row-contiguous sources are read with
+// the lanes along the rows into a shared tile.  Either way a lane splits and writes two
+// consecutive K elements.  The bound is HBM (8 bytes read and NS slices written per
+// element); what keeps the kernel from it is instructions, so none of them is FP64 and the
+// offsets take 32-bit divisions.
 constexpr int PK_R = 32, PK_K = 128;
 
 // destinations of the NS slices of a packed operand
@@ -821,37 +847,34 @@ struct PackDst {
   void* p[3];
 };
 
+// Splits the floats nearest to two K elements (their 24 bits hold more than hi + lo keep; hi +
+// mid + lo of bf16 keep all of them; each residual is exact in float) and stores the slices
+// at o, o + 1 (o even).
 template <int PREC, int NS>
-__device__ __forceinline__ void pack_store(const PackDst& dst, int64_t o, double x) {
-  // split the float nearest to x (its 24 bits hold more than hi + lo keep; hi + mid + lo of
-  // bf16 keep all of them); each residual is exact in float
-  const float f = d2f_bits(x);
+__device__ __forceinline__ void pack_store2(const PackDst& dst, int64_t o, float f0, float f1) {
   if (PREC == 1) {
-    const float h = tf32_rna(f);
-    const float l = tf32_rna(__fsub_rn(f, h));
-    reinterpret_cast<float*>(dst.p[0])[o] = h;
-    reinterpret_cast<float*>(dst.p[1])[o] = l;
+    const float h0 = tf32_rna(f0), h1 = tf32_rna(f1);
+    *reinterpret_cast<float2*>(reinterpret_cast<float*>(dst.p[0]) + o) = make_float2(h0, h1);
+    *reinterpret_cast<float2*>(reinterpret_cast<float*>(dst.p[1]) + o) =
+        make_float2(tf32_rna(__fsub_rn(f0, h0)), tf32_rna(__fsub_rn(f1, h1)));
   } else {
-    const __nv_bfloat16 h = __float2bfloat16_rn(f);
-    const float r = __fsub_rn(f, __bfloat162float(h));
-    const __nv_bfloat16 m = __float2bfloat16_rn(r);
-    reinterpret_cast<__nv_bfloat16*>(dst.p[0])[o] = h;
-    reinterpret_cast<__nv_bfloat16*>(dst.p[1])[o] = m;
-    if (NS == 3) reinterpret_cast<__nv_bfloat16*>(dst.p[2])[o] = __float2bfloat16_rn(__fsub_rn(r, __bfloat162float(m)));
+    const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+    const float r0 = __fsub_rn(f0, __low2float(h)), r1 = __fsub_rn(f1, __high2float(h));
+    const __nv_bfloat162 m = __floats2bfloat162_rn(r0, r1);
+    *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(dst.p[0]) + o) = h;
+    *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(dst.p[1]) + o) = m;
+    if (NS == 3)
+      *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(dst.p[2]) + o) =
+          __floats2bfloat162_rn(__fsub_rn(r0, __low2float(m)), __fsub_rn(r1, __high2float(m)));
   }
 }
 
 // GEN: the operand is the Gaussian sketch whose element index is the offset the modes
 // give (philox.cuh, float Box-Muller); src is not read.
-template <int PREC, bool GEN>
-__device__ __forceinline__ double operand_at(const double* __restrict__ src, const GaussSrc& gs,
-                                             int64_t off) {
-  if (GEN) {
-    float z0, z1;
-    gauss_pair_f32(gs.seed, gs.sid, gs.replica, off >> 1, z0, z1);
-    return double((off & 1) ? z1 : z0);
-  }
-  return __ldg(src + off);
+__device__ __forceinline__ float sketch_at(const GaussSrc& gs, int64_t off) {
+  float z0, z1;
+  gauss_pair_f32(gs.seed, gs.sid, gs.replica, off >> 1, z0, z1);
+  return (off & 1) ? z1 : z0;
 }
 
 template <int PREC, int NS, bool GEN>
@@ -859,87 +882,100 @@ __global__ void __launch_bounds__(256) pack_kernel(const double* __restrict__ sr
                                                    DevModes km, int64_t R, int64_t K, int64_t Kp,
                                                    int64_t ktiles, int64_t ntiles, PackDst dst,
                                                    int r_contig, GaussSrc gs) {
-  __shared__ int64_t roff[PK_R], koff[PK_K];
-  __shared__ double tile[PK_R][PK_K + 1];
+  __shared__ int64_t roff[PK_R];
+  __shared__ __align__(16) int64_t koff[PK_K];
+  __shared__ __align__(8) float tile[GEN ? 1 : PK_R][PK_K + 2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;  // 8 warps
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int64_t r0 = (t / ktiles) * PK_R, k0 = (t % ktiles) * PK_K;
     __syncthreads();  // the previous strip is done with roff, koff and tile
     if (tid < PK_R) {
-      int64_t a = 0, b = 0;
-      if (r0 + tid < R) mode_offsets(rm, r0 + tid, a, b);
-      roff[tid] = a;
+      roff[tid] = r0 + tid < R ? src_offset32(rm, uint32_t(r0 + tid)) : 0;
     } else if (tid < PK_R + PK_K) {
       const int j = tid - PK_R;
-      int64_t a = 0, b = 0;
-      if (k0 + j < K) mode_offsets(km, k0 + j, a, b);
-      koff[j] = a;
+      koff[j] = k0 + j < K ? src_offset32(km, uint32_t(k0 + j)) : 0;
     }
     __syncthreads();
     if (GEN) {
       // generated sketch: warp w takes the row pairs (2w, 2w + 1), (2w + 16, 2w + 17); when
       // the two rows hold consecutive sketch elements 2c, 2c + 1 (the row mode is the
       // innermost one), one Philox call gives both
-#pragma unroll
+#pragma unroll 1
       for (int i = 0; i < PK_R / 16; ++i) {
         const int rr = 2 * (warp + 8 * i);
         const int64_t r = r0 + rr;
+#pragma unroll 1
+        for (int j = 0; j < PK_K / 64; ++j) {
+          const int kk = 2 * lane + 64 * j;
+          if (k0 + kk >= Kp) continue;
+          float v[2][2];
 #pragma unroll
-        for (int j = 0; j < PK_K / 32; ++j) {
-          const int kk = lane + 32 * j;
-          const int64_t k = k0 + kk;
-          if (k >= Kp) continue;
-          double v0 = 0.0, v1 = 0.0;
-          if (k < K) {
-            const int64_t o0 = roff[rr] + koff[kk], o1 = roff[rr + 1] + koff[kk];
-            if (r < R && r + 1 < R && o1 == o0 + 1 && (o0 & 1) == 0) {
-              float z0, z1;
-              gauss_pair_f32(gs.seed, gs.sid, gs.replica, o0 >> 1, z0, z1);
-              v0 = double(z0);
-              v1 = double(z1);
-            } else {
-              if (r < R) v0 = operand_at<PREC, true>(src, gs, o0);
-              if (r + 1 < R) v1 = operand_at<PREC, true>(src, gs, o1);
+          for (int c = 0; c < 2; ++c) {
+            v[0][c] = v[1][c] = 0.0f;
+            if (k0 + kk + c < K) {
+              const int64_t o0 = roff[rr] + koff[kk + c], o1 = roff[rr + 1] + koff[kk + c];
+              if (r + 1 < R && o1 == o0 + 1 && (o0 & 1) == 0) {
+                gauss_pair_f32(gs.seed, gs.sid, gs.replica, o0 >> 1, v[0][c], v[1][c]);
+              } else {
+                if (r < R) v[0][c] = sketch_at(gs, o0);
+                if (r + 1 < R) v[1][c] = sketch_at(gs, o1);
+              }
             }
           }
-          pack_store<PREC, NS>(dst, r * Kp + k, v0);
-          pack_store<PREC, NS>(dst, (r + 1) * Kp + k, v1);
+          pack_store2<PREC, NS>(dst, r * Kp + k0 + kk, v[0][0], v[0][1]);
+          pack_store2<PREC, NS>(dst, (r + 1) * Kp + k0 + kk, v[1][0], v[1][1]);
         }
       }
     } else if (!r_contig) {
-      // warp w: rows w, w + 8, ...; lanes along K (coalesced reads and writes)
+      // warp w: rows w, w + 8, ...; a lane reads two consecutive K elements
 #pragma unroll
-      for (int i = 0; i < PK_R / 8; ++i) {
-        const int rr = warp + 8 * i;
-        const int64_t r = r0 + rr;
-        double v[PK_K / 32];
+      for (int i = 0; i < PK_R / 8; i += 2) {
+        double v[2][PK_K / 64][2];
 #pragma unroll
-        for (int j = 0; j < PK_K / 32; ++j) {
-          const int kk = lane + 32 * j;
-          v[j] = (r < R && k0 + kk < K) ? operand_at<PREC, GEN>(src, gs, roff[rr] + koff[kk]) : 0.0;
+        for (int i2 = 0; i2 < 2; ++i2) {
+          const int rr = warp + 8 * (i + i2);
+#pragma unroll
+          for (int j = 0; j < PK_K / 64; ++j) {
+            const int kk = 2 * lane + 64 * j;
+            const longlong2 ko = *reinterpret_cast<const longlong2*>(koff + kk);
+            const double* const p = src + roff[rr];
+            v[i2][j][0] = (r0 + rr < R && k0 + kk < K) ? __ldg(p + ko.x) : 0.0;
+            v[i2][j][1] = (r0 + rr < R && k0 + kk + 1 < K) ? __ldg(p + ko.y) : 0.0;
+          }
         }
 #pragma unroll
-        for (int j = 0; j < PK_K / 32; ++j) {
-          const int64_t k = k0 + lane + 32 * j;
-          if (k < Kp) pack_store<PREC, NS>(dst, r * Kp + k, v[j]);
-        }
+        for (int i2 = 0; i2 < 2; ++i2)
+#pragma unroll
+          for (int j = 0; j < PK_K / 64; ++j) {
+            const int64_t k = k0 + 2 * lane + 64 * j;
+            if (k < Kp)
+              pack_store2<PREC, NS>(dst, (r0 + warp + 8 * (i + i2)) * Kp + k, d2f_bits(v[i2][j][0]), d2f_bits(v[i2][j][1]));
+          }
       }
     } else {
       // lanes along the rows for the reads (the source is contiguous in r)
+      const bool in = r0 + lane < R;
+      const double* const p = src + roff[lane];
 #pragma unroll
-      for (int i = 0; i < PK_K / 8; ++i) {
-        const int kk = warp + 8 * i;
-        const bool ok = (r0 + lane < R) && (k0 + kk < K);
-        tile[lane][kk] = ok ? operand_at<PREC, GEN>(src, gs, roff[lane] + koff[kk]) : 0.0;
+      for (int i = 0; i < PK_K / 8; i += 8) {
+        double v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int kk = warp + 8 * (i + c);
+          v[c] = (in && k0 + kk < K) ? __ldg(p + koff[kk]) : 0.0;
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) tile[lane][warp + 8 * (i + c)] = d2f_bits(v[c]);
       }
       __syncthreads();
 #pragma unroll
       for (int i = 0; i < PK_R / 8; ++i) {
         const int rr = warp + 8 * i;
 #pragma unroll
-        for (int j = 0; j < PK_K / 32; ++j) {
-          const int64_t k = k0 + lane + 32 * j;
-          if (k < Kp) pack_store<PREC, NS>(dst, (r0 + rr) * Kp + k, tile[rr][lane + 32 * j]);
+        for (int j = 0; j < PK_K / 64; ++j) {
+          const int kk = 2 * lane + 64 * j;
+          const float2 f = *reinterpret_cast<const float2*>(&tile[rr][kk]);
+          if (k0 + kk < Kp) pack_store2<PREC, NS>(dst, (r0 + rr) * Kp + k0 + kk, f.x, f.y);
         }
       }
     }
@@ -1081,14 +1117,10 @@ __global__ void __launch_bounds__(256) oz_exp_kernel(const double* __restrict__ 
     const int64_t r0 = (t / ktiles) * PK_R, k0 = (t % ktiles) * PK_K;
     __syncthreads();
     if (tid < PK_R) {
-      int64_t a = 0, c = 0;
-      if (r0 + tid < R) mode_offsets(rm, r0 + tid, a, c);
-      roff[tid] = a;
+      roff[tid] = r0 + tid < R ? src_offset32(rm, uint32_t(r0 + tid)) : 0;
     } else if (tid < PK_R + PK_K) {
       const int j = tid - PK_R;
-      int64_t a = 0, c = 0;
-      if (k0 + j < K) mode_offsets(km, k0 + j, a, c);
-      koff[j] = a;
+      koff[j] = k0 + j < K ? src_offset32(km, uint32_t(k0 + j)) : 0;
     }
     __syncthreads();
     if (r_contig) {  // lane = row; warp w takes K elements w, w + 8, ...
@@ -1134,15 +1166,11 @@ __global__ void __launch_bounds__(256) oz_pack_kernel(const double* __restrict__
     const int64_t r0 = (t / ktiles) * PK_R, k0 = (t % ktiles) * PK_K;
     __syncthreads();
     if (tid < PK_R) {
-      int64_t a = 0, c = 0;
-      if (r0 + tid < R) mode_offsets(rm, r0 + tid, a, c);
-      roff[tid] = a;
+      roff[tid] = r0 + tid < R ? src_offset32(rm, uint32_t(r0 + tid)) : 0;
       rexp[tid] = r0 + tid < R ? exps[r0 + tid] : OZ_EXP_NONE;
     } else if (tid < PK_R + PK_K) {
       const int j = tid - PK_R;
-      int64_t a = 0, c = 0;
-      if (k0 + j < K) mode_offsets(km, k0 + j, a, c);
-      koff[j] = a;
+      koff[j] = k0 + j < K ? src_offset32(km, uint32_t(k0 + j)) : 0;
     }
     __syncthreads();
     if (!r_contig) {
