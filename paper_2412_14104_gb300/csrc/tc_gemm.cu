@@ -105,6 +105,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
 }
 __device__ __forceinline__ bool all_lanes(bool p) { return __all_sync(0xffffffffu, p) != 0; }
+// One lane of the (converged) warp, as the TMA and MMA branches choose it: the compiler knows
+// that such a branch runs with one lane and keeps descriptors and addresses in uniform
+// registers; under `lane == 0` it moved every operand of every MMA there, which took the
+// issuing thread longer than the tensor core needs (96 MMAs of a 3xTF32 stage sequence
+// 5.8 us, 4.2 with elect.sync, 3.0 at the peak rate).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred a;\n elect.sync _|a, 0xffffffff;\n selp.u32 %0, 1, 0, a;\n}\n" : "=r"(p));
+  return p != 0;
+}
 // CTA pairs (a cluster of two CTAs on two SMs sharing one MMA)
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -620,7 +630,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
   const uint32_t tmem = tmem_base_s;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;  // stage uses, continued across units
       bool ok = true;
       for (int u = first; u < units && ok; u += stride) {
@@ -658,7 +668,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
         mbar_wait(&full_bar[i % STAGES], (i / STAGES) & 1);
     }
   } else if (warp == 1 && (!PAIR || rank == 0)) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t id = idesc<PREC, PAIR ? 2 * TC_BM : TC_BM, BN>();
       int it = 0, cc = 0;  // stage uses and chunks, continued across units
       bool ok = true;
@@ -704,7 +714,7 @@ __global__ void __maxnreg__(96)  // 18 warps x 96 registers fit one SM's registe
       mbar_wait<PAIR>(&fin_bar, 0);
     }
   } else if (warp == 1) {  // PAIR, rank 1
-    if (lane == 0) {
+    if (elect_one()) {
       // second CTA of a pair: forward "stage landed" to the first CTA, which issues the MMAs
       const uint32_t peer0 = cluster_addr(&peer_full[0], 0);
       int it = 0;
@@ -1269,7 +1279,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
   const uint32_t tmem = tmem_base_s;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool ok = true;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
@@ -1290,7 +1300,7 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
       for (int i = max(0, it - OZ_STAGES); i < it; ++i) mbar_wait(&full_bar[i % OZ_STAGES], (i / OZ_STAGES) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t id = idesc<2, TC_BM, OZ_BN>();
       int it = 0, cc = 0;
       bool ok = true;
