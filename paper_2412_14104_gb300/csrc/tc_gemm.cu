@@ -1303,38 +1303,47 @@ __global__ void __maxnreg__(96) oz_gemm_kernel(const __grid_constant__ OzMaps ma
     if (elect_one()) {
       constexpr uint32_t id = idesc<2, TC_BM, OZ_BN>();
       int it = 0, cc = 0;
-      bool ok = true;
+      // This thread waits for what comes next (the stage that follows, at the end of a chunk
+      // the other accumulators) while half of the stage's 30 MMAs are still to be issued:
+      // between two stages there is the commit alone (451 -> 406 us for the chi = 24 C2; the
+      // 12 to 24 MMAs of a tc_gemm_kernel stage leave less to hide behind, and it was slower).
+      auto landed = [&](int n) {
+        const bool there = mbar_wait(&full_bar[n % OZ_STAGES], (n / OZ_STAGES) & 1);
+        tc_fence_after();
+        return there;
+      };
+      auto drained = [&](int n) {
+        const bool free = n < 2 || mbar_wait(&acc_empty[n & 1], (n / 2 - 1) & 1);
+        tc_fence_after();
+        return free;
+      };
+      const uint64_t desc = sdesc_sw64(smem_u32(smem));
+      bool ok = int(blockIdx.x) >= units || landed(0);
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const Unit w = oz_unit_of(g, u);
-        const int nchunks = (w.nk + OZ_KC - 1) / OZ_KC;
-        for (int c = 0; c < nchunks && ok; ++c, ++cc) {
-          const int b = cc & 1, use = cc >> 1;
-          if (use > 0 && !mbar_wait(&acc_empty[b], (use - 1) & 1)) { ok = false; break; }
-          tc_fence_after();
+        const bool last = u + int(gridDim.x) >= units;
+        for (int i = 0; i < w.nk && ok; ++i, ++it) {
+          const int s = it % OZ_STAGES, b = cc & 1;
+          const bool begins = i % OZ_KC == 0, ends = i % OZ_KC == OZ_KC - 1 || i + 1 == w.nk;
           const uint32_t acc = tmem + uint32_t(b * ACC_COLS);
-          const int i_end = min(w.nk, (c + 1) * OZ_KC);
-          for (int i = c * OZ_KC; i < i_end; ++i, ++it) {
-            const int s = it % OZ_STAGES, round = it / OZ_STAGES;
-            if (!mbar_wait(&full_bar[s], round & 1)) { ok = false; break; }
-            tc_fence_after();
-            const uint64_t d0 = sdesc_sw64(smem_u32(smem + s * OZ_STAGE));
-            uint64_t ad[OZ_NS], bd[OZ_NS];
+          const uint64_t d0 = desc + uint64_t(s * (OZ_STAGE >> 4));
 #pragma unroll
-            for (int p = 0; p < OZ_NS; ++p) {
-              ad[p] = d0 + uint64_t((p * OZ_A_TILE) >> 4);
-              bd[p] = d0 + uint64_t((OZ_NS * OZ_A_TILE + p * OZ_B_TILE) >> 4);
+          for (int kk = 0; kk < OZ_KS / 32; ++kk) {  // 16 bf16 of K per instruction
+            if (kk == OZ_KS / 64) {
+              if (i + 1 < w.nk || !last) ok = landed(it + 1);
+              if (ends && !(last && i + 1 == w.nk)) ok = drained(cc + 1) && ok;
             }
 #pragma unroll
-            for (int kk = 0; kk < OZ_KS / 32; ++kk) {  // 16 bf16 of K per instruction
-              const uint64_t off = uint64_t(kk * 2);
-#pragma unroll
-              for (int t = 0; t < 15; ++t)
-                mma<2, 1>(acc + uint32_t(oz_acc(t) * OZ_BN), ad[oz_a(t)] + off, bd[oz_b(t)] + off, id,
-                          (i > c * OZ_KC || kk > 0 || !oz_first(t)) ? 1u : 0u);
-            }
-            mma_commit<1>(&empty_bar[s]);
+            for (int t = 0; t < 15; ++t)
+              mma<2, 1>(acc + uint32_t(oz_acc(t) * OZ_BN), d0 + uint64_t(((oz_a(t) * OZ_A_TILE) >> 4) + 2 * kk),
+                        d0 + uint64_t(((OZ_NS * OZ_A_TILE + oz_b(t) * OZ_B_TILE) >> 4) + 2 * kk), id,
+                        (!begins || kk > 0 || !oz_first(t)) ? 1u : 0u);
           }
-          if (ok) mma_commit<1>(&acc_full[b]);
+          mma_commit<1>(&empty_bar[s]);
+          if (ends) {
+            mma_commit<1>(&acc_full[b]);
+            ++cc;
+          }
         }
       }
       mma_commit<1>(&fin_bar);
