@@ -195,9 +195,12 @@ __global__ void __launch_bounds__(256) chol_inverse_kernel(const double* G, int 
 // R_ii, each warp summing every fourth term, in the order of a 32-lane butterfly.  Operations
 // and their order are those of a textbook Cholesky and substitution (near_*: see there).
 //
-// Bound by two FP64 chains of about 1000 and 750 clocks a row: 11 us at n = 12, where one
-// block of 1024 threads and a warp per column of the inverse took 18 + 12 us and a host read
-// of the status between them.
+// Bound by two FP64 chains a row.  An FP64 instruction holds a warp's port for 64 clocks also
+// when it is predicated off, so the rows of four that are done, or that n <= 4 U does not
+// have, are left out at compile time: 26 -> 17 us at n = 12, 63 -> 49 at n = 30 (one block of
+// 1024 threads and a warp per column of the inverse took 18 + 12 us and a host read of the
+// status between them at n = 12, and had other bits).
+template <int U>
 __global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G, int n, double* R, double* X,
                                                                  int* status, int first, double shift_rel) {
   __shared__ double Rs[32][33], Xs[32][33], part[2][4][32], inv[32];
@@ -212,9 +215,9 @@ __global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G
     thr[lane] = ref > 0.0 ? __double_as_longlong(1e-14 * ref) : 0x7FF0000000000000ll;
     if (lane == 0) fail_s = 0;
   }
-  double v[8];
+  double v[U];  // row 4 u + warp
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int i = 4 * u + warp;
     v[u] = (i < n && lane >= i && lane < n) ? G[i * n + lane] + (i == lane ? sh : 0.0) : 0.0;
     Rs[i][lane] = 0.0;
@@ -222,16 +225,18 @@ __global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G
   }
   __syncthreads();
   bool fail = false;
-  for (int j0 = 0; j0 < n && !fail; j0 += 4) {  // v[u] is row j0 + 4 u + warp
-    for (int w = 0; w < 4 && j0 + w < n; ++w) {
-      const int j = j0 + w;
+#pragma unroll
+  for (int b = 0; b < U; ++b) {
+#pragma unroll 1
+    for (int w = 0; w < 4 && 4 * b + w < n && !fail; ++w) {
+      const int j = 4 * b + w;
       if (warp == w) {
-        const double d = __shfl_sync(0xffffffffu, v[0], j);
+        const double d = __shfl_sync(0xffffffffu, v[b], j);
         const int ex = exponent_field(d);
         const bool bad = !(__double_as_longlong(d) > thr[j]) || ex == 0 || ex >= 2044;
         double h;
         const double root = near_sqrt(bad ? 1.0 : d, h), r = near_rcp_pivot(root, 2.0 * h);
-        if (lane >= j) Rs[j][lane] = lane == j ? root : near_div(v[0], root, r);
+        if (lane >= j) Rs[j][lane] = lane == j ? root : near_div(v[b], root, r);
         if (lane == j) {
           inv[j] = r;
           if (bad) fail_s = 1;
@@ -242,20 +247,20 @@ __global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G
       if (fail) break;
       const double g = Rs[j][lane];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = j0 + 4 * u + warp;
+      for (int u = b; u < U; ++u) {
+        const int i = 4 * u + warp;
         if (i > j && i < n) v[u] = fma(-Rs[j][i], g, v[u]);
       }
     }
-#pragma unroll
-    for (int u = 0; u < 7; ++u) v[u] = v[u + 1];
   }
-  if (!fail) {
-    for (int i = n - 1; i >= 0; --i) {
-      const int cnt = n - 1 - i;  // terms k = i + 1 + l, l < cnt; this warp's are l = 4 t + warp
-      double pr[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
+  for (int b = 0; b < U; ++b) {  // rows with 4 b .. 4 b + 3 terms
+#pragma unroll 1
+    for (int w = 0; w < 4 && 4 * b + w < n && !fail; ++w) {
+      const int cnt = 4 * b + w, i = n - 1 - cnt;  // terms k = i + 1 + l, l < cnt; this warp's are l = 4 t + warp
+      double pr[U];
+#pragma unroll
+      for (int t = 0; t <= b; ++t) {
         const int l = 4 * t + warp;
         pr[t] = 0.0;
         if (l < cnt) pr[t] = __dmul_rn(Rs[i][i + 1 + l], Xs[i + 1 + l][lane]);  // not fused into the sum
@@ -264,7 +269,7 @@ __global__ void __launch_bounds__(128) chol_inverse_small_kernel(const double* G
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
-        for (int t = 0; t < o; ++t)
+        for (int t = 0; t < o && t + o <= b; ++t)
           if (4 * (t + o) + warp < cnt) pr[t] += pr[t + o];
       part[i & 1][warp][lane] = pr[0];
       __syncthreads();
@@ -1327,7 +1332,10 @@ void cholesky_inverse(const double* G, int n, double* R, double* Rinv, int* stat
   check_extent(Rinv, int64_t(n) * n - 1, sizeof(double), "cholesky inverse");
   TATRG_CHECK(n >= 1 && n <= kCholMaxN, TATRG_EINVAL, "cholesky: n must be <= 168");
   if (n <= 32) {
-    chol_inverse_small_kernel<<<1, 128, 0, s>>>(G, n, R, Rinv, status_dev, first ? 1 : 0, shift_rel);
+    const auto k = n <= 8 ? chol_inverse_small_kernel<2> : n <= 12 ? chol_inverse_small_kernel<3>
+                 : n <= 16 ? chol_inverse_small_kernel<4> : n <= 24 ? chol_inverse_small_kernel<6>
+                                                        : chol_inverse_small_kernel<8>;
+    k<<<1, 128, 0, s>>>(G, n, R, Rinv, status_dev, first ? 1 : 0, shift_rel);
     TATRG_CUDA(cudaGetLastError());
   } else if (n <= 64) launch_chol<4>(G, n, R, Rinv, status_dev, first, shift_rel, s);
   else launch_chol<8>(G, n, R, Rinv, status_dev, first, shift_rel, s);
