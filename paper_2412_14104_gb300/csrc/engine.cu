@@ -111,26 +111,27 @@ int Engine::read_flag(int idx) {
 
 // CholeskyQR2 (Yamamoto et al. 2015), optionally with a shifted first pass (shifted
 // CholeskyQR3, Fukaya et al. 2020): Q = Y R^-1, R = R2 R1.  ok = false on breakdown.
-OrthResult Engine::cholqr2(const double* Y, int64_t m, int64_t n, double shift, bool& ok) {
+OrthResult Engine::cholqr2(const double* Y, int64_t m, int64_t n, double shift, bool want_r, bool& ok) {
   OrthResult out;
   const int passes = shift > 0.0 ? 3 : 2;
-  DevBuf G(n * n * sizeof(double), s_), Rk(n * n * sizeof(double), s_),
-      Ri(n * n * sizeof(double), s_), Racc(n * n * sizeof(double), s_),
-      Rtmp(n * n * sizeof(double), s_);
+  DevBuf G(n * n * sizeof(double), s_), Rk(n * n * sizeof(double), s_), Ri(n * n * sizeof(double), s_), Racc, Rtmp;
+  if (want_r) {
+    Racc.alloc(n * n * sizeof(double), s_);
+    Rtmp.alloc(n * n * sizeof(double), s_);
+  }
   DMat cur;
   const double* src = Y;
   for (int pass = 0; pass < passes; ++pass) {
     mm(n, n, m, src, n, true, src, n, false, G.d(), n);
-    cholesky_inverse(G.d(), int(n), Rk.d(), Ri.d(), flag(0), pass == 0, pass == 0 ? shift : 0.0, s_);
+    cholesky_inverse(G.d(), int(n), want_r && pass == 0 ? Racc.d() : Rk.d(), Ri.d(), flag(0), pass == 0,
+                     pass == 0 ? shift : 0.0, s_);
     st_.launches++;
     DMat nxt;
     nxt.buf = dalloc(m * n, s_);
     nxt.rows = m;
     nxt.cols = n;
     mm(m, n, n, src, n, false, Ri.d(), n, false, nxt.p(), n);
-    if (pass == 0) {
-      TATRG_CUDA(cudaMemcpyAsync(Racc.d(), Rk.d(), n * n * sizeof(double), cudaMemcpyDeviceToDevice, s_));
-    } else {
+    if (want_r && pass > 0) {
       mm(n, n, n, Rk.d(), n, false, Racc.d(), n, false, Rtmp.d(), n);
       std::swap(Racc, Rtmp);
     }
@@ -141,21 +142,23 @@ OrthResult Engine::cholqr2(const double* Y, int64_t m, int64_t n, double shift, 
   ok = read_flag(0) == 0;
   if (!ok) return out;
   out.Q = std::move(cur);
-  out.R.buf = std::move(Racc);
-  out.R.rows = n;
-  out.R.cols = n;
+  if (want_r) {
+    out.R.buf = std::move(Racc);
+    out.R.rows = n;
+    out.R.cols = n;
+  }
   out.k = int(n);
   return out;
 }
 
-OrthResult Engine::orth(const double* Y, int64_t m, int64_t n) {
+OrthResult Engine::orth(const double* Y, int64_t m, int64_t n, bool want_r) {
   TATRG_CHECK(n >= 1, TATRG_EINVAL, "orth: empty matrix");
   bool ok = false;
   OrthResult r;
   if (m >= n && n <= cholesky_max_n()) {
     // FP64 Grams: plain CholeskyQR2.  Split-precision Grams carry ~1e-7 relative error, so
     // their first pass is shifted (shifted CholeskyQR3).
-    r = cholqr2(Y, m, n, fp64_grade() ? 0.0 : 1e-6, ok);
+    r = cholqr2(Y, m, n, fp64_grade() ? 0.0 : 1e-6, want_r, ok);
     if (ok) return r;
   }
   // Rank-revealing fallback: one-sided Jacobi SVD of Y itself (no squared condition
@@ -179,47 +182,49 @@ OrthResult Engine::orth(const double* Y, int64_t m, int64_t n) {
   return out;
 }
 
-Engine::MetricOrth Engine::orth_metric(const double* X, int64_t nin, int64_t w, const Op& metric) {
+Engine::MetricOrth Engine::orth_metric(const double* X, int64_t nin, int64_t w, const Op& metric, bool want_r) {
   MetricOrth out;
   if (w > cholesky_max_n()) return out;  // ok = false: the caller takes the explicit path
   const int passes = fp64_grade() ? 2 : 3;
   const double shift = fp64_grade() ? 0.0 : 1e-6;
-  DevBuf G(w * w * sizeof(double), s_), Rk(w * w * sizeof(double), s_), Ri(w * w * sizeof(double), s_),
-      Racc(w * w * sizeof(double), s_), Rtmp(w * w * sizeof(double), s_);
+  DevBuf G(w * w * sizeof(double), s_), Rk(w * w * sizeof(double), s_), Ri(w * w * sizeof(double), s_), Racc, Rtmp;
+  if (want_r) {
+    Racc.alloc(w * w * sizeof(double), s_);
+    Rtmp.alloc(w * w * sizeof(double), s_);
+  }
   DMat cur;
-  cur.buf = dalloc(nin * w, s_);
-  cur.rows = nin;
-  cur.cols = w;
-  TATRG_CUDA(cudaMemcpyAsync(cur.p(), X, nin * w * sizeof(double), cudaMemcpyDeviceToDevice, s_));
+  const double* src = X;
   DMat U;
   U.buf = dalloc(nin * w, s_);
   U.rows = nin;
   U.cols = w;
   for (int pass = 0; pass < passes; ++pass) {
-    metric(cur.p(), w, U.p());
-    mm(w, w, nin, cur.p(), w, true, U.p(), w, false, G.d(), w);
-    cholesky_inverse(G.d(), int(w), Rk.d(), Ri.d(), flag(0), pass == 0, pass == 0 ? shift : 0.0, s_);
+    metric(src, w, U.p());
+    mm(w, w, nin, src, w, true, U.p(), w, false, G.d(), w);
+    cholesky_inverse(G.d(), int(w), want_r && pass == 0 ? Racc.d() : Rk.d(), Ri.d(), flag(0), pass == 0,
+                     pass == 0 ? shift : 0.0, s_);
     st_.launches++;
     DMat nxt;
     nxt.buf = dalloc(nin * w, s_);
     nxt.rows = nin;
     nxt.cols = w;
-    mm(nin, w, w, cur.p(), w, false, Ri.d(), w, false, nxt.p(), w);
-    if (pass == 0) {
-      TATRG_CUDA(cudaMemcpyAsync(Racc.d(), Rk.d(), w * w * sizeof(double), cudaMemcpyDeviceToDevice, s_));
-    } else {
+    mm(nin, w, w, src, w, false, Ri.d(), w, false, nxt.p(), w);
+    if (want_r && pass > 0) {
       mm(w, w, w, Rk.d(), w, false, Racc.d(), w, false, Rtmp.d(), w);
       std::swap(Racc, Rtmp);
     }
     cur = std::move(nxt);
+    src = cur.p();
   }
   if (read_flag(0) != 0) return out;  // a breakdown in some pass: ok = false
   metric(cur.p(), w, U.p());  // U = G V for the final basis
   out.V = std::move(cur);
   out.U = std::move(U);
-  out.R.buf = std::move(Racc);
-  out.R.rows = w;
-  out.R.cols = w;
+  if (want_r) {
+    out.R.buf = std::move(Racc);
+    out.R.rows = w;
+    out.R.cols = w;
+  }
   out.k = int(w);
   out.ok = true;
   return out;
@@ -268,16 +273,16 @@ SvdResult Engine::rsvd(const Op& apply, const Op& rapply, int64_t rows, int64_t 
   DMat Y;
   Y.buf = dalloc(rows * ell, s_);
   apply(omega, ell, Y.p());
-  OrthResult Q = orth(Y.p(), rows, ell);
+  OrthResult Q = orth(Y.p(), rows, ell, false);
   for (int it = 0; it < q; ++it) {
     DMat Z;
     Z.buf = dalloc(cols * Q.k, s_);
     rapply(Q.Q.p(), Q.k, Z.p());
-    OrthResult Qt = orth(Z.p(), cols, Q.k);
+    OrthResult Qt = orth(Z.p(), cols, Q.k, false);
     DMat Y2;
     Y2.buf = dalloc(rows * Qt.k, s_);
     apply(Qt.Q.p(), Qt.k, Y2.p());
-    Q = orth(Y2.p(), rows, Qt.k);
+    Q = orth(Y2.p(), rows, Qt.k, false);
   }
   DMat Bt;
   Bt.buf = dalloc(cols * Q.k, s_);
@@ -310,16 +315,16 @@ SvdResult Engine::rsvd_psd(const double* rho, int64_t n, int64_t ell, int q, con
   DMat Y;
   Y.buf = dalloc(n * ell, s_);
   app(omega, ell, Y.p());
-  OrthResult Q = orth(Y.p(), n, ell);
+  OrthResult Q = orth(Y.p(), n, ell, false);
   for (int it = 0; it < q; ++it) {
     DMat Z;
     Z.buf = dalloc(n * Q.k, s_);
     app(Q.Q.p(), Q.k, Z.p());
-    OrthResult Qt = orth(Z.p(), n, Q.k);
+    OrthResult Qt = orth(Z.p(), n, Q.k, false);
     DMat Y2;
     Y2.buf = dalloc(n * Qt.k, s_);
     app(Qt.Q.p(), Qt.k, Y2.p());
-    Q = orth(Y2.p(), n, Qt.k);
+    Q = orth(Y2.p(), n, Qt.k, false);
   }
   const int64_t k = Q.k;
   DMat RQ;

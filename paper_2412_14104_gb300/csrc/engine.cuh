@@ -52,7 +52,9 @@ class Engine {
           const double* B, int64_t ldb, bool tb, double* C, int64_t ldc, double alpha = 1.0,
           double beta = 0.0);
 
-  OrthResult orth(const double* Y, int64_t m, int64_t n);
+  // want_r = false: R is left empty (a subspace iteration needs the basis alone, and R takes a
+  // product and two buffers in each pass)
+  OrthResult orth(const double* Y, int64_t m, int64_t n, bool want_r = true);
   SvdResult svd(const double* A, int64_t m, int64_t n);
 
   // Randomized SVD of an implicit rows x cols operator: apply(X, w, Y) computes
@@ -74,7 +76,7 @@ class Engine {
     int k = 0;
     bool ok = false;
   };
-  MetricOrth orth_metric(const double* X, int64_t nin, int64_t w, const Op& metric);
+  MetricOrth orth_metric(const double* X, int64_t nin, int64_t w, const Op& metric, bool want_r = true);
 
   // Forward-mode (tangent) rules, in tangent.cu.  grp[i] is the multiplet id of singular
   // value i: pairs inside one multiplet get no mutual rotation.
@@ -108,7 +110,7 @@ class Engine {
   double* scratch_double() { return reinterpret_cast<double*>(flag_.as<int>() + 2); }
 
  private:
-  OrthResult cholqr2(const double* Y, int64_t m, int64_t n, double shift, bool& ok);
+  OrthResult cholqr2(const double* Y, int64_t m, int64_t n, double shift, bool want_r, bool& ok);
   cudaStream_t s_;
   Stats st_;
   DevBuf flag_;

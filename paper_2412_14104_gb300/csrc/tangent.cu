@@ -194,7 +194,7 @@ Engine::SvdTan Engine::svd_tan(const double* Ad, int64_t m, int64_t n, const Svd
 Engine::OrthT Engine::orth_t(const double* Y, const double* Yd, int64_t m, int64_t n, double tau) {
   OrthT out;
   bool ok = false;
-  if (m >= n) out.o = cholqr2(Y, m, n, 0.0, ok);
+  if (m >= n) out.o = cholqr2(Y, m, n, 0.0, true, ok);
   if (ok) {
     DevBuf Ri(n * n * sizeof(double), s_), C(n * n * sizeof(double), s_), X(n * n * sizeof(double), s_);
     tri_inverse(out.o.R.p(), int(n), Ri.d(), s_);

@@ -709,13 +709,13 @@ void tatrg_ctx::rg_step() {
         }
       }
       om.release();
-      Engine::MetricOrth Qm = eng.orth_metric(W0.p(), nL, ell, metric_L);
+      Engine::MetricOrth Qm = eng.orth_metric(W0.p(), nL, ell, metric_L, false);
       bool ok = Qm.ok;
       for (int it = 0; ok && it < p.q; ++it) {
-        Engine::MetricOrth Qt = eng.orth_metric(Qm.U.p(), nL, ell, metric_R);
+        Engine::MetricOrth Qt = eng.orth_metric(Qm.U.p(), nL, ell, metric_R, false);
         ok = Qt.ok;
         if (ok) {
-          Qm = eng.orth_metric(Qt.U.p(), nL, ell, metric_L);
+          Qm = eng.orth_metric(Qt.U.p(), nL, ell, metric_L, false);
           ok = Qm.ok;
         }
       }
