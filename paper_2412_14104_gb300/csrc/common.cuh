@@ -81,8 +81,8 @@ void trim_block_memory();
 // from the library's own pool of the current device, which keeps up to 2 GiB between calls.
 // The default pool returns everything at each synchronisation unless a context has told it
 // not to, and mapping it again costs more than many calls compute: 1.2 ms of a 2.96 ms
-// chi = 32 contraction in 3xTF32 (0.55 GB of packed operands), 0.2 of 0.67 ms at chi = 24,
-// 45 us of a 363 us SVD.  2 GiB holds the operands of every contraction up to chi = 38;
+// chi = 32 contraction in 3xTF32 (0.55 GB of packed operands), 0.3 of 0.67 ms at chi = 24,
+// 0.09 of an orthonormalisation's 0.87.  2 GiB holds the operands of every contraction up to chi = 38;
 // above that the call computes for far longer than it maps.
 class BlockMemory {
  public:
