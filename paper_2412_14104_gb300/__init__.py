@@ -367,7 +367,7 @@ def set_cta_pairs(mode):
 
 def release_memory():
     """Gives the working memory that the building-block calls keep (at most 2 GiB on each
-    device) back to the driver."""
+    device) back."""
     _check(lib().tatrg_release_memory())
 
 

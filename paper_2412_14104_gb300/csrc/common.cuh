@@ -74,7 +74,7 @@ inline void check_extent(const void* p, int64_t max_elem, size_t esize, const ch
 // The pool that this thread's allocations come from: nullptr, the device's default pool, or
 // inside a building-block call (BlockMemory, engine.cu) the library's own.
 cudaMemPool_t& thread_pool();
-// Gives the free memory of the library's own pools back to the driver (all devices).
+// Unmaps the free memory of the library's own pools (all devices).
 void trim_block_memory();
 
 // For the duration of a building-block call outside a context, the calling thread allocates

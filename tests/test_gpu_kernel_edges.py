@@ -163,7 +163,7 @@ def test_split_contraction_sums_two_floats_exactly(torch, prec, mode):
 
 
 def test_block_memory_is_bounded_and_given_back(torch):
-    """The building blocks' pool: at most 2 GiB (and the driver's granularity) kept after a call
+    """The building blocks' pool: at most 2 GiB (and the mapping granularity) kept after a call
     that used 2.4 GB, nothing after release_memory(), and calls of two threads on two streams."""
     import threading
     M, N, K = 65536, 256, 4608  # 2.4 GB of packed operands in 3xTF32
